@@ -4,19 +4,16 @@
 // centres are binned into a uniform grid whose cell width is the diameter of
 // the largest bounding sphere (slightly enlarged so rounding cannot separate
 // an overlapping pair by more than one cell) -- of the largest one below a cut
-// that leaves at most big_cap oversized pills out of the cells, which are then
-// paired from their own side against the cells in their reach and against
-// each other (a stretched outlier would otherwise coarsen the whole grid).
-// The grid is built with a
-// count / exclusive-scan / scatter pass that also copies each pill's sphere
-// and group into cell order.  Candidate pairs are then built in parallel (the
-// paper's extension of Green's particle grid): one warp per cell holds the
-// cell's pills one per lane and tests them against the pills of the cell
-// itself and of its 13 forward neighbours (each neighbouring pair of cells
-// is visited once), staged 32 at a time in shared memory; hits are compacted
-// with __ballot_sync / __popc and output slots reserved with one atomic per
-// step.  The pair order inside the list is not fixed, the pair set is; every
-// consumer is order independent.
+// that leaves at most big_cap oversized pills, which are paired from their own
+// side against the cells in their reach (a stretched outlier would otherwise
+// coarsen the whole grid).  The grid is built with a count / exclusive-scan /
+// scatter pass that also copies each pill's sphere and group into cell order.
+// Candidate pairs are then built in parallel (the paper's extension of Green's
+// particle grid): a thread per pill tests the pills of its own cell after it
+// and those of the 13 forward neighbours (each neighbouring pair of cells is
+// visited once); a warp's hits are gathered in shared memory and written
+// together, one atomic reserving their slots.  The pair order inside the list
+// is not fixed, the pair set is; every consumer is order independent.
 //
 // Contact handling (Sec. 7, Sec. 7.2): each candidate pair runs the
 // dichotomous narrowphase and, if the pills interpenetrate, one XPBD update of
@@ -34,25 +31,37 @@ constexpr int kBpThreads = 256;  // choose_cut takes two histogram bins per thre
 __global__ void __launch_bounds__(kBpThreads) bp_bounds_kernel(Params P)
 {
     __shared__ int hist[kRadBins];
+    __shared__ unsigned int s_bounds[8];
     for (int b = threadIdx.x; b < kRadBins; b += blockDim.x) hist[b] = 0;
+    if (threadIdx.x < 8) s_bounds[threadIdx.x] = 0u;
     __syncthreads();
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY}, mr = 0.f;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.ns; g += gridDim.x * blockDim.x) {
-        const float4 sp = bp_sphere(P, g);
-        P.spheres[g] = sp;
+    const int lane = threadIdx.x & 31;
+    for (int g0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); g0 < P.ns; g0 += gridDim.x * blockDim.x) {
+        const unsigned in = __ballot_sync(0xffffffffu, g0 + lane < P.ns);
+        if (g0 + lane >= P.ns) continue;
+        const float4 sp = bp_sphere(P, g0 + lane);
+        P.spheres[g0 + lane] = sp;
         mn[0] = fminf(mn[0], sp.x); mn[1] = fminf(mn[1], sp.y); mn[2] = fminf(mn[2], sp.z);
         mx[0] = fmaxf(mx[0], sp.x); mx[1] = fmaxf(mx[1], sp.y); mx[2] = fmaxf(mx[2], sp.z);
         mr = fmaxf(mr, sp.w);
-        atomicAdd(hist + rad_bin(sp.w), 1);
+        // most pills of a scene share a few bins: one addition per bin and warp
+        const int bin = rad_bin(sp.w);
+        const unsigned peers = __match_any_sync(in, bin);
+        if (lane == __ffs(peers) - 1) atomicAdd(hist + bin, __popc(peers));
     }
-    merge_bounds(P, mn, mx, mr);
+    __syncwarp();
+    merge_bounds_to(s_bounds, mn, mx, mr);
     __syncthreads();
+    // one merge per block: the seven words are single addresses of the whole grid
+    // (a merge per warp took 17 of this kernel's 25 us at 300,000 pills)
+    if (threadIdx.x < 7 && s_bounds[threadIdx.x]) atomicMax(P.bounds + threadIdx.x, s_bounds[threadIdx.x]);
     for (int b = threadIdx.x; b < kRadBins; b += blockDim.x)
         if (hist[b]) atomicAdd(P.bp_hist + b, hist[b]);
 }
 
 // Grid for this substep (the cut radius from the histogram, the same in every
-// block); pills above the cut go to the oversized list instead of a cell.
+// block); pills above the cut are listed as well.
 __global__ void __launch_bounds__(kBpThreads) bp_count_kernel(Params P)
 {
     __shared__ int sh[kRadBins + 33];
@@ -65,17 +74,16 @@ __global__ void __launch_bounds__(kBpThreads) bp_count_kernel(Params P)
         *P.npairs = 0;  // pair cursor of bp_emit_kernel
         if (!ok) atomicOr(P.err, ERR_NONFINITE);
     }
+    const unsigned int big = big_threshold(G.b_cut);
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.ns; g += gridDim.x * blockDim.x) {
         const float4 sp = P.spheres[g];
-        if (rad_bin(sp.w) > G.b_cut) {
-            P.cell_of[g] = -1;
+        if (__float_as_uint(sp.w) > big) {
             const int slot = atomicAdd(P.bp_hist + kRadBins, 1);
             if (slot < P.big_cap) P.big_list[slot] = g;
-        } else {
-            const int cell = bp_cell(G, sp);
-            P.cell_of[g] = cell;
-            atomicAdd(P.cell_count + cell, 1);
         }
+        const int cell = bp_cell(G, sp);
+        P.cell_of[g] = cell;
+        atomicAdd(P.cell_count + cell, 1);
     }
 }
 
@@ -84,24 +92,24 @@ __global__ void bp_scatter_kernel(Params P)
 {
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.ns; g += gridDim.x * blockDim.x) {
         const int cell = P.cell_of[g];
-        if (cell >= 0) scatter_pill(P, g, cell, P.cell_start[cell]);
+        scatter_pill(P, g, cell, P.cell_start[cell]);
     }
 }
 
-// Pair search: a thread per grid pill in cell order (emit_pills), then a warp
-// per oversized pill (emit_big).
+// Pair search: a warp per oversized pill (emit_big), then a thread per pill in
+// cell order (emit_pills).
 constexpr int kEmitWarps = 8;
 __global__ void __launch_bounds__(32 * kEmitWarps, 4) bp_emit_kernel(Params P)
 {
-    __shared__ int2 buf[kEmitWarps][kPairBuf];
+    __shared__ int buf[kEmitWarps][kEmitBuf];
     const Grid G = *P.grid;
     if (G.pad) return;  // no valid grid: no candidates
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int warp = blockIdx.x * kEmitWarps + wib, nwarps = gridDim.x * kEmitWarps;
-    const int n_grid = P.cell_start[grid_cells(P.grid, P.table)];  // pills in the cells
-    emit_pills(P, G, n_grid, warp, nwarps, buf[wib], lane);
+    const unsigned int big = big_threshold(G.b_cut);
     const int nb = min(P.bp_hist[kRadBins], P.big_cap);
-    for (int i = warp; i < nb; i += nwarps) emit_big(P, G, i, nb, lane);
+    for (int i = warp; i < nb; i += nwarps) emit_big(P, G, big, i, buf[wib], lane);
+    emit_pills(P, G, big, warp, nwarps, buf[wib], lane);
 }
 
 // ---------------------------------------------------------------- exclusive scan

@@ -896,8 +896,8 @@ __device__ __forceinline__ void merge_bounds(const Params &P, float mn[3], float
 // thousands of pills in each cell.  The multi-kernel broadphase therefore
 // histograms the radii (16 bins per octave: the float's exponent and top four
 // mantissa bits) and sizes the cell for the cut radius below which all but at
-// most big_cap pills lie; the pills above it stay out of the cells and are
-// paired from their own side (bp_big_kernel).  The pair set is unchanged:
+// most big_cap pills lie.  The pills above it sit in the cells like the others
+// but are paired from their own side (emit_big).  The pair set is unchanged:
 // every candidate is still decided by spheres_overlap.
 constexpr unsigned int kRadBinBase = (127u - 20u) << 4;  // bin 0 starts at 2^-20
 __device__ __forceinline__ int rad_bin(float R)
@@ -907,6 +907,13 @@ __device__ __forceinline__ int rad_bin(float R)
 }
 // Upper edge of bin b (exclusive): every radius of bins <= b is below it.
 __device__ __forceinline__ float rad_bin_top(int b) { return __uint_as_float(((unsigned)b + 1u + kRadBinBase) << 19); }
+
+// Oversized pills are those with rad_bin(R) > b_cut: the bits of R, as an
+// unsigned number, above this threshold (none when b_cut is the last bin).
+__device__ __forceinline__ unsigned int big_threshold(int b_cut)
+{
+    return b_cut < kRadBins - 1 ? (((unsigned)b_cut + 1u + kRadBinBase) << 19) - 1u : 0xffffffffu;
+}
 
 // Cut bin from the histogram, by every thread of a 256-thread block (the same
 // result in every block): the smallest b such that bins above b hold at most
@@ -1042,148 +1049,173 @@ __device__ __forceinline__ void emit_cell(const Params &P, const Grid &G, int u,
     }
 }
 
-// Writes the warp's hits (lane: pair (a, b) when `hit`) as (lower id, higher
-// id) with their segments' first vertices and zero multipliers, reserving the
-// output slots with one atomic.  Every lane of the warp calls it.
-__device__ __forceinline__ void emit_warp_hits(const Params &P, bool hit, int a, int b, int lane)
+// ---------------------------------------------------------------- pair search of large scenes
+// Hits wait in the warp's shared buffer as cell-order entries: kLanePairs a
+// lane, rows one word apart modulo the banks, so that appending (a row per
+// lane) and flushing (along rows) are both free of bank conflicts.
+constexpr int kLanePairs = 24, kLaneRow = kLanePairs + 1, kEmitBuf = 32 * kLaneRow;
+
+// Writes pair number idx of pills (a, first vertex va) and (b, vb) as (lower id, higher id).
+__device__ __forceinline__ void put_pair(const Params &P, int idx, int a, int va, int b, int vb)
+{
+    if (idx >= P.max_pairs) return;
+    if (P.pairs) P.pairs[idx] = make_int2(min(a, b), max(a, b));
+    if (P.pair_v) P.pair_v[idx] = a < b ? make_int2(va, vb) : make_int2(vb, va);
+    if (P.lam_pair) P.lam_pair[idx] = 0.f;
+}
+
+// Flushes the lanes' rows (cnt hits in this lane's, found for pill ia with
+// first vertex va) with one atomic and coalesced stores, row after row: the
+// pairs of one pill stay together in the list, so that lanes of the contact
+// pass share its vertices.  Output t belongs to the last row that starts at or
+// before t.  Every lane of the warp calls it.
+__device__ __forceinline__ void flush_rows(const Params &P, const int *buf, int cnt, int ia, int va, int lane)
 {
     const unsigned full = 0xffffffffu;
-    const unsigned hm = __ballot_sync(full, hit);
-    if (!hm) return;
-    int out = 0;
-    if (lane == 0) out = atomicAdd(P.npairs, __popc(hm));
-    out = __shfl_sync(full, out, 0);
-    if (hit) {
-        const int idx = out + __popc(hm & ((1u << lane) - 1u));
-        if (idx < P.max_pairs) {
-            const int lo = min(a, b), hi = max(a, b);
-            P.pairs[idx] = make_int2(lo, hi);
-            if (P.pair_v) P.pair_v[idx] = make_int2(P.seg_v0[lo], P.seg_v0[hi]);
-            if (P.lam_pair) P.lam_pair[idx] = 0.f;
+    const int inc = warp_incl_scan(cnt), off = inc - cnt;
+    const int total = __shfl_sync(full, inc, 31);
+    int base = 0;
+    if (lane == 0) base = atomicAdd(P.npairs, total);
+    base = __shfl_sync(full, base, 0);
+    __syncwarp();
+    for (int t0 = 0; t0 < total; t0 += 32) {
+        const int t = min(t0 + lane, total - 1);
+        int l = 0;
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1)
+            if (__shfl_sync(full, off, l + s) <= t) l += s;
+        const int k = t - __shfl_sync(full, off, l);
+        const int a = __shfl_sync(full, ia, l), v = __shfl_sync(full, va, l);
+        if (t0 + lane < total) {
+            const int b = P.cell_pills[buf[l * kLaneRow + k]];
+            put_pair(P, base + t, a, v, b, P.pair_v ? P.seg_v0[b] : 0);
         }
+    }
+    __syncwarp();
+}
+
+// spheres_overlap with the components in packed pairs (add and multiply two
+// floats at a time, each rounded as the scalar operation): (b - a) and, in the
+// fourth place, Ra + Rb, then their squares.  na = (-ax, -ay, -az, Ra).
+__device__ __forceinline__ bool spheres_overlap2(float4 na, float4 b)
+{
+    float ex, ey, ez, rs;
+    asm("{\n\t.reg .b64 p, q, r, s;\n\t"
+        "mov.b64 p, {%4, %5};\n\tmov.b64 q, {%6, %7};\n\t"
+        "mov.b64 r, {%8, %9};\n\tmov.b64 s, {%10, %11};\n\t"
+        "add.rn.f32x2 p, p, r;\n\tadd.rn.f32x2 q, q, s;\n\t"
+        "mul.rn.f32x2 p, p, p;\n\tmul.rn.f32x2 q, q, q;\n\t"
+        "mov.b64 {%0, %1}, p;\n\tmov.b64 {%2, %3}, q;\n\t}"
+        : "=f"(ex), "=f"(ey), "=f"(ez), "=f"(rs)
+        : "f"(na.x), "f"(na.y), "f"(na.z), "f"(na.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w));
+    return __fadd_rn(__fadd_rn(ex, ey), ez) <= rs;
+}
+
+// Candidate pairs of the pills up to the cut, a thread per pill in cell order
+// (lane: entry p of the cell-order copies, pills p0 .. p0 + 31 per warp step).
+// Each tests the pills of its own cell after it and those of the 13 forward
+// neighbour cells (dz = 1; dz = 0, dy = 1; dz = dy = 0, dx = 1), so every pair
+// of pills in neighbouring cells is tested once.  Cells are numbered along x,
+// so these are five runs of the cell order: the rest of the own cell with the
+// next one, and four rows of three cells.  A lane walks its runs end to end,
+// four candidates a step; the warp takes the longest lane's number of steps.
+// Settled strands (300,000 pills, 8.8 million pairs): 216 us a search with the
+// oversized pills, against 469 us with fourteen lists each walked to the warp's
+// longest and the oversized pills tested against their whole list.
+__device__ __forceinline__ void emit_pills(const Params &P, const Grid &G, unsigned int big, int warp, int nwarps,
+                                           int *buf, int lane)
+{
+    const unsigned full = 0xffffffffu;
+    int *row = buf + lane * kLaneRow;
+    for (int p0 = warp * 32; p0 < P.ns; p0 += nwarps * 32) {
+        const int p = p0 + lane;
+        float4 na = make_float4(0.f, 0.f, 0.f, 0.f);
+        int ga = 0, ia = 0, va = 0, cnt = 0;
+        int q = 0, end = 0, q1 = 0, e1 = 0, q2 = 0, e2 = 0, q3 = 0, e3 = 0, q4 = 0, e4 = 0;
+        if (p < P.ns) {
+            const float4 sa = P.cell_sph[p];
+            if (!(__float_as_uint(sa.w) > big)) {
+                na = make_float4(-sa.x, -sa.y, -sa.z, sa.w);
+                ga = P.cell_grp[p];
+                ia = P.cell_pills[p];
+                const int ix = cell_coord(sa.x, G.lo[0], G.inv_cell, G.dim[0]);
+                const int iy = cell_coord(sa.y, G.lo[1], G.inv_cell, G.dim[1]);
+                const int iz = cell_coord(sa.z, G.lo[2], G.inv_cell, G.dim[2]);
+                const int x0 = max(ix - 1, 0), x1 = min(ix + 1, G.dim[0] - 1) + 1;
+                const int r0 = G.dim[0] * (iy + G.dim[1] * iz), ry = G.dim[0], rz = G.dim[0] * G.dim[1];
+                const int *cs = P.cell_start;
+                const bool up = iy + 1 < G.dim[1], down = iy > 0, next = iz + 1 < G.dim[2];
+                q = p + 1;
+                end = cs[r0 + x1];
+                if (up) { q1 = cs[r0 + ry + x0]; e1 = cs[r0 + ry + x1]; }
+                if (next && down) { q2 = cs[r0 + rz - ry + x0]; e2 = cs[r0 + rz - ry + x1]; }
+                if (next) { q3 = cs[r0 + rz + x0]; e3 = cs[r0 + rz + x1]; }
+                if (next && up) { q4 = cs[r0 + rz + ry + x0]; e4 = cs[r0 + rz + ry + x1]; }
+                if (P.pair_v) va = P.seg_v0[ia];
+            }
+        }
+        int left = 4;  // runs after the current one
+        while (true) {
+            while (q >= end && left > 0) {
+                q = q1; end = e1;
+                q1 = q2; e1 = e2;
+                q2 = q3; e2 = e3;
+                q3 = q4; e3 = e4;
+                --left;
+            }
+            if (!__any_sync(full, q < end)) break;
+            float4 cs[4];
+            int cg[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (q + t < end) {
+                    cs[t] = P.cell_sph[q + t];
+                    cg[t] = P.cell_grp[q + t];
+                }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (q + t < end && cg[t] != ga && spheres_overlap2(na, cs[t]) && !(__float_as_uint(cs[t].w) > big))
+                    row[cnt++] = q + t;
+            q += 4;
+            if (__any_sync(full, cnt > kLanePairs - 4)) {
+                flush_rows(P, buf, cnt, ia, va, lane);
+                cnt = 0;
+            }
+        }
+        if (__any_sync(full, cnt > 0)) flush_rows(P, buf, cnt, ia, va, lane);
     }
 }
 
-// Candidate pairs of the grid's pills, a thread per pill in cell order
-// (lane: entry p of the cell-order copies, pills p0 .. p0 + 31 per warp step):
-// each tests the pills of its own cell after it and those of the 13 forward
-// neighbour cells (dz = 1; dz = 0, dy = 1; dz = dy = 0, dx = 1), so every pair
-// of pills in neighbouring cells is tested once.  Consecutive lanes mostly
-// share a cell, hence the same neighbour lists (their loads are broadcasts).
-// Each list is walked for the warp's longest length (shorter lanes idle), so
-// that every step ends with one ballot: hits go to the warp's shared buffer
-// buf (kPairBuf pairs), which is flushed to the pair list with one atomic.
-// 480 pairs (3.75 KB per warp): one flush atomic per 480 pairs, measured 2 % faster than 160
-// on the hair; after a flush it holds one step's hits (at most 4 x 32)
-constexpr int kPairBuf = 480;
-
-__device__ __forceinline__ void flush_pairs(const Params &P, const int2 *buf, int cnt, int lane)
+__device__ __forceinline__ void flush_big(const Params &P, const int *buf, int cnt, int ia, int va, int lane)
 {
-    __syncwarp();
     int base = 0;
     if (lane == 0) base = atomicAdd(P.npairs, cnt);
     base = __shfl_sync(0xffffffffu, base, 0);
+    __syncwarp();
     for (int t = lane; t < cnt; t += 32) {
-        const int idx = base + t;
-        if (idx < P.max_pairs) {
-            const int2 pr = buf[t];
-            const int lo = min(pr.x, pr.y), hi = max(pr.x, pr.y);
-            P.pairs[idx] = make_int2(lo, hi);
-            if (P.pair_v) P.pair_v[idx] = make_int2(P.seg_v0[lo], P.seg_v0[hi]);
-            if (P.lam_pair) P.lam_pair[idx] = 0.f;
-        }
+        const int b = P.cell_pills[buf[t]];
+        put_pair(P, base + t, ia, va, b, P.pair_v ? P.seg_v0[b] : 0);
     }
     __syncwarp();
 }
 
-__device__ __forceinline__ void emit_pills(const Params &P, const Grid &G, int n_grid, int warp, int nwarps,
-                                           int2 *buf, int lane)
+// Candidate pairs of oversized pill i of the list, by one warp: all pills up to
+// the cut, and of the oversized ones those that come after it in the order of
+// descending radius (equal radii by id), so that each pair is found once, from
+// its larger pill, and lies within |Ri| + max(|Ri|, r_cut) of its centre.  The
+// cells of that box (enlarged by 2^-8 for the rounding of its corners) are rows
+// of the cell order; 32 rows' ends are loaded at a time.  (Radii can be
+// negative: contacts squeeze them past zero; their bits then sort above every
+// cut.)
+__device__ __forceinline__ void emit_big(const Params &P, const Grid &G, unsigned int big, int i, int *buf, int lane)
 {
     const unsigned full = 0xffffffffu;
-    int cnt = 0;  // pairs in buf (uniform over the warp)
-    for (int p0 = warp * 32; p0 < n_grid; p0 += nwarps * 32) {
-        const int p = p0 + lane;
-        const bool own = p < n_grid;
-        float4 sa = make_float4(0.f, 0.f, 0.f, 0.f);
-        int ga = 0, ia = 0, ix = 0, iy = 0, iz = 0;
-        if (own) {
-            sa = P.cell_sph[p];
-            ga = P.cell_grp[p];
-            ia = P.cell_pills[p];
-            ix = cell_coord(sa.x, G.lo[0], G.inv_cell, G.dim[0]);
-            iy = cell_coord(sa.y, G.lo[1], G.inv_cell, G.dim[1]);
-            iz = cell_coord(sa.z, G.lo[2], G.inv_cell, G.dim[2]);
-        }
-        for (int k = 0; k < 14; ++k) {
-            int d0 = 0, d1 = 0;
-            if (own) {
-                int dx = 0, dy = 0, dz = 0;
-                if (k < 9) {
-                    dx = k % 3 - 1; dy = k / 3 - 1; dz = 1;
-                } else if (k < 12) {
-                    dx = k - 10; dy = 1;
-                } else if (k == 12) {
-                    dx = 1;
-                }
-                const int x = ix + dx, y = iy + dy, z = iz + dz;
-                if (x >= 0 && x < G.dim[0] && y >= 0 && y < G.dim[1] && z < G.dim[2]) {
-                    const int d = x + G.dim[0] * (y + G.dim[1] * z);
-                    d0 = k == 13 ? p + 1 : P.cell_start[d];
-                    d1 = P.cell_start[d + 1];
-                }
-            }
-            const int len = d1 - d0;
-            const int steps = __reduce_max_sync(full, len > 0 ? len : 0);
-            // four candidates per step: their loads are issued before any test
-            for (int j = 0; j < steps; j += 4) {
-                float4 cs[4];
-                int cg[4];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int q = d0 + j + t;
-                    if (j + t < len) {
-                        cs[t] = P.cell_sph[q];
-                        cg[t] = P.cell_grp[q];
-                    }
-                }
-                unsigned m[4];
-                bool hit[4];
-                int nh = 0;
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    hit[t] = j + t < len && cg[t] != ga && spheres_overlap(sa, cs[t]);
-                    m[t] = __ballot_sync(full, hit[t]);
-                    nh += __popc(m[t]);
-                }
-                if (nh) {
-                    if (cnt + nh > kPairBuf) {
-                        flush_pairs(P, buf, cnt, lane);
-                        cnt = 0;
-                    }
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        if (hit[t]) buf[cnt + __popc(m[t] & ((1u << lane) - 1u))] = make_int2(ia, P.cell_pills[d0 + j + t]);
-                        cnt += __popc(m[t]);
-                    }
-                }
-            }
-        }
-    }
-    if (cnt) flush_pairs(P, buf, cnt, lane);
-}
-
-// Candidate pairs of oversized pill i of the list (bounding radius above the
-// grid's cut), by one warp: (1) against the pills in the cells of the box
-// centre +- (R_i + r_cut)(1 + 2^-8) -- a grid pill overlapping pill i has its
-// centre within R_i + r_cut, and the enlargement covers the rounding of the
-// box corners -- tested 32 at a time from the cell-order copies; (2) against
-// the oversized pills after i in the list, so that each pair is found once.
-__device__ __forceinline__ void emit_big(const Params &P, const Grid &G, int i, int nb, int lane)
-{
     const int gi = P.big_list[i];
     const float4 si = P.spheres[gi];
-    const int grp = P.seg_group[gi];
-    const float reach = __fmul_rn(__fadd_rn(si.w, G.r_cut), 1.00390625f);
+    const float4 na = make_float4(-si.x, -si.y, -si.z, si.w);
+    const float Ri = fabsf(si.w);
+    const int grp = P.seg_group[gi], vi = P.pair_v ? P.seg_v0[gi] : 0;
+    const float reach = __fmul_rn(__fadd_rn(Ri, fmaxf(Ri, G.r_cut)), 1.00390625f);
     const float c[3] = {si.x, si.y, si.z};
     int lo[3], hi[3];
 #pragma unroll
@@ -1191,32 +1223,43 @@ __device__ __forceinline__ void emit_big(const Params &P, const Grid &G, int i, 
         lo[k] = cell_coord(__fsub_rn(c[k], reach), G.lo[k], G.inv_cell, G.dim[k]);
         hi[k] = cell_coord(__fadd_rn(c[k], reach), G.lo[k], G.inv_cell, G.dim[k]);
     }
-    for (int z = lo[2]; z <= hi[2]; ++z)
-        for (int y = lo[1]; y <= hi[1]; ++y) {
-            // the cells x = lo .. hi of one row are contiguous in cell order
+    const int ny = hi[1] - lo[1] + 1, rows = ny * (hi[2] - lo[2] + 1);
+    int cnt = 0;  // hits in buf (uniform over the warp)
+    for (int rb = 0; rb < rows; rb += 32) {
+        int s0 = 0, s1 = 0;
+        if (rb + lane < rows) {
+            const int y = lo[1] + (rb + lane) % ny, z = lo[2] + (rb + lane) / ny;
             const int row = G.dim[0] * (y + G.dim[1] * z);
-            const int p0 = P.cell_start[row + lo[0]], p1 = P.cell_start[row + hi[0] + 1];
+            s0 = P.cell_start[row + lo[0]];
+            s1 = P.cell_start[row + hi[0] + 1];
+        }
+        const int nr = min(32, rows - rb);
+        for (int r = 0; r < nr; ++r) {
+            const int p0 = __shfl_sync(full, s0, r), p1 = __shfl_sync(full, s1, r);
             for (int pb = p0; pb < p1; pb += 32) {
                 const int q = pb + lane;
                 bool hit = false;
-                int b = 0;
                 if (q < p1) {
-                    hit = P.cell_grp[q] != grp && spheres_overlap(si, P.cell_sph[q]);
-                    if (hit) b = P.cell_pills[q];
+                    const float4 sj = P.cell_sph[q];
+                    hit = P.cell_grp[q] != grp && spheres_overlap2(na, sj);
+                    if (hit && __float_as_uint(sj.w) > big) {
+                        const float Rj = fabsf(sj.w);
+                        hit = Rj < Ri || (Rj == Ri && P.cell_pills[q] < gi);
+                    }
                 }
-                emit_warp_hits(P, hit, gi, b, lane);
+                const unsigned m = __ballot_sync(full, hit);
+                if (hit) buf[cnt + __popc(m & ((1u << lane) - 1u))] = q;
+                cnt += __popc(m);
+                if (cnt > kEmitBuf - 32) {
+                    __syncwarp();
+                    flush_big(P, buf, cnt, gi, vi, lane);
+                    cnt = 0;
+                }
             }
         }
-    for (int j0 = i + 1; j0 < nb; j0 += 32) {
-        const int j = j0 + lane;
-        bool hit = false;
-        int b = 0;
-        if (j < nb) {
-            b = P.big_list[j];
-            hit = P.seg_group[b] != grp && spheres_overlap(si, P.spheres[b]);
-        }
-        emit_warp_hits(P, hit, gi, b, lane);
     }
+    __syncwarp();
+    if (cnt) flush_big(P, buf, cnt, gi, vi, lane);
 }
 
 // The chunk's pills (lane: entry pa of the cell order, sphere sa, group ga,
