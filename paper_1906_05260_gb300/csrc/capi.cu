@@ -758,7 +758,7 @@ size_t viper_scene_footprint(const viper_scene_desc *d)
             size_t table = (size_t)next_pow2(std::max<long long>(2LL * (long long)ns, 4096));
             b += 20 * cap + 16 * ns + 4 * (2 * ns) + 4 * (2 * table + 1) + 4 * 4096;  // pairs, their vertices, lambda
             b += 4 * (kBoundsWords + (size_t)broadphase_big_cap((int)ns));  // radius histogram, oversized pills
-            b += 16 * nv;  // world pack
+            b += (16 + 32) * nv;  // world and pill packs
             b += 16 * (ns + ns / 32 + 1);  // pair-search chunk records
         }
     }
@@ -936,7 +936,7 @@ int viper_scene_create(const viper_scene_desc *d, viper_scene **out)
     A(s->d_scan_tmp, 4096);
     A(P.bar, 4); A(P.tile_sums, 1024);
     A(P.contact_stats, pills ? 3 : 1);
-    A(s->xw, pills ? nv : 1);
+    A(s->xw, pills ? nv : 1); A(s->pb, pills ? 2 * (size_t)nv : 1);
 #undef A
 #undef AC
     cudaMemsetAsync(P.err, 0, sizeof(int), s->stream);

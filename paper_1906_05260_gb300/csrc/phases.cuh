@@ -109,6 +109,19 @@ __device__ __forceinline__ float4 world_pack(const Params &P, int v, float4 x)
     return make_float4(__fadd_rn(x.x, o.x), __fadd_rn(x.y, o.y), __fadd_rn(x.z, o.z), __fmul_rn(x.w, P.RV0[v].w));
 }
 
+// The pill between world-packed vertices a and b for the early-out of the
+// contact pass: box[0] = (midpoint, r), box[1] = (axis d = b - a, |d|^2), r the
+// larger radius padded by 1e-3 of itself and 1e-5 of the coordinates' and the
+// axis's magnitude, far above the FP32 rounding of the early-out or the search.
+__device__ __forceinline__ void pill_box(float4 a, float4 b, float4 *box)
+{
+    const V3 d = xyz(b) - xyz(a), m = 0.5f * (xyz(a) + xyz(b));
+    const float r = fmaxf(a.w, b.w), dd = dot(d, d);
+    const float mag = fmaxf(fmaxf(fabsf(m.x), fabsf(m.y)), fabsf(m.z)) + fabsf(d.x) + fabsf(d.y) + fabsf(d.z);
+    box[0] = make_float4(m.x, m.y, m.z, r + 1e-3f * fabsf(r) + 1e-5f * mag);
+    box[1] = make_float4(d.x, d.y, d.z, dd);
+}
+
 __device__ __forceinline__ float4 to_world(const Params &P, int v, float4 x)
 {
     float4 o = P.rod_origin[P.rod_of_v[v]];
@@ -654,7 +667,12 @@ __device__ __forceinline__ void rod_item(const Params &P, int b, int n_iter, boo
             check_finite(P, x);
         }
         P.X[v] = x;
-        if (P.XW) P.XW[v] = world_pack(P, v, x);
+        if (P.XW) {
+            const float4 xw = world_pack(P, v, x);
+            P.XW[v] = xw;
+            // the pill from v on (after a rod's last vertex: not a pill, and not read)
+            if (i + 1 < item.y) pill_box(xw, world_pack(P, v + 1, sX[i + 1]), P.PB + 2 * (size_t)v);
+        }
     }
     for (int j = threadIdx.x; j < item.w; j += blockDim.x) {
         const int g = item.z + j;
@@ -1443,16 +1461,20 @@ struct ContactPair {
     float rbar[4];  // their rest radii
 };
 
+// World positions and radii packed by the preceding sweep: the pair's first
+// vertices pv and four 16-byte gathers (rest radii: only if active).
+__device__ __forceinline__ void contact_load_packed(const Params &P, int2 pv, ContactPair &c)
+{
+    const float4 xa1 = P.XW[pv.x], xa2 = P.XW[pv.x + 1], xb1 = P.XW[pv.y], xb2 = P.XW[pv.y + 1];
+    c.vs[0] = pv.x; c.vs[1] = pv.x + 1; c.vs[2] = pv.y; c.vs[3] = pv.y + 1;
+    c.Q.a1 = xyz(xa1); c.Q.a2 = xyz(xa2); c.Q.b1 = xyz(xb1); c.Q.b2 = xyz(xb2);
+    c.Q.ra1 = xa1.w; c.Q.ra2 = xa2.w; c.Q.rb1 = xb1.w; c.Q.rb2 = xb2.w;
+}
+
 __device__ __forceinline__ void contact_load(const Params &P, int i, ContactPair &c)
 {
     if (P.XW) {
-        // world positions and radii packed by the preceding sweep: the pair's
-        // first vertices and four 16-byte gathers (rest radii: only if active)
-        const int2 pv = P.pair_v[i];
-        const float4 xa1 = P.XW[pv.x], xa2 = P.XW[pv.x + 1], xb1 = P.XW[pv.y], xb2 = P.XW[pv.y + 1];
-        c.vs[0] = pv.x; c.vs[1] = pv.x + 1; c.vs[2] = pv.y; c.vs[3] = pv.y + 1;
-        c.Q.a1 = xyz(xa1); c.Q.a2 = xyz(xa2); c.Q.b1 = xyz(xb1); c.Q.b2 = xyz(xb2);
-        c.Q.ra1 = xa1.w; c.Q.ra2 = xa2.w; c.Q.rb1 = xb1.w; c.Q.rb2 = xb2.w;
+        contact_load_packed(P, P.pair_v[i], c);
         return;
     }
     const int2 pr = P.pairs[i];
@@ -1567,6 +1589,39 @@ __device__ __forceinline__ bool contact_may_touch(const PillPair &Q)
     return !sat_separated(n, e, da, db, lim);
 }
 
+// The same certificate from the pills' packs (pill_box), for the pass over many
+// pairs: with e the line through the midpoints, the closest points e + s da - t db,
+// s, t in [-1/2, 1/2], by alternating clamped minima (approximate divisions: any
+// direction n gives a valid bound, and the padding covers the bound's own
+// rounding; a NaN or infinite n certifies nothing).  One 256-bit load per
+// pill and about 65 operations; from the four vertices, with IEEE divisions and
+// square roots, the test took 350 instructions a warp.
+__device__ __forceinline__ void ld_pill_box(const float4 *b, float4 &m, float4 &d)
+{
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(m.x), "=f"(m.y), "=f"(m.z), "=f"(m.w), "=f"(d.x), "=f"(d.y), "=f"(d.z), "=f"(d.w)
+        : "l"(b));
+}
+
+__device__ __forceinline__ bool boxes_may_touch(const Params &P, int2 pv)
+{
+    float4 am, ad, bm, bd;
+    ld_pill_box(P.PB + 2 * (size_t)pv.x, am, ad);
+    ld_pill_box(P.PB + 2 * (size_t)pv.y, bm, bd);
+    const V3 e = xyz(am) - xyz(bm), da = xyz(ad), db = xyz(bd);
+    const float lim = am.w + bm.w;
+    const float ee = dot(e, e), ea = dot(e, da), eb = dot(e, db);
+    if (ee - 0.5f * (fabsf(ea) + fabsf(eb)) > lim * sqrt_approx(ee)) return false;
+    const float ab = dot(da, db);
+    const float den = ad.w * bd.w - ab * ab;
+    const float s0 = den > 1e-6f * ad.w * bd.w ? fminf(fmaxf(fdiv(ab * eb - bd.w * ea, den), -0.5f), 0.5f) : 0.f;
+    const float t = fminf(fmaxf(fdiv(ab * s0 + eb, bd.w), -0.5f), 0.5f);
+    const float s = fminf(fmaxf(fdiv(ab * t - ea, ad.w), -0.5f), 0.5f);
+    const V3 n = e + s * da - t * db;
+    const float gap = fabsf(dot(n, e)) - 0.5f * (fabsf(dot(n, da)) + fabsf(dot(n, db)));
+    return !(gap > lim * sqrt_approx(dot(n, n)));
+}
+
 // Pair i by one thread.
 __device__ __forceinline__ void contact_pair(const Params &P, int i, float at)
 {
@@ -1592,35 +1647,57 @@ __device__ __forceinline__ int contact_pair_warp(const Params &P, int i, float a
 }
 
 // Pairs [0, np) a thread each, by the calling warp from chunk `chunk` of 32
-// pairs on, every `stride`-th chunk.  The pairs that may touch
-// (contact_may_touch) are queued in the warp's buffer q (64 ints of shared
-// memory) and searched 32 at a time, so that the search runs on full warps
-// however sparse the touching pairs are.  Same results as contact_pair.
-// Returns the warp's counts (searched, active), the same in every lane.
+// pairs on, every `stride`-th chunk.  The pairs that may touch are queued in
+// the warp's buffer q (64 pairs of shared memory) and searched 32 at a time,
+// so that the search runs on full warps however sparse the touching pairs are.
+// The next chunk's pairs are loaded before this one is tested.  Same results
+// as contact_pair.  Returns the warp's counts (searched, active), the same in
+// every lane.
+struct QueuedPair {
+    int i;
+    int2 v;
+};
+
+__device__ __forceinline__ bool queued_contact(const Params &P, QueuedPair j, float at)
+{
+    ContactPair c;
+    if (P.XW)
+        contact_load_packed(P, j.v, c);
+    else
+        contact_load(P, j.i, c);
+    pill_pair_axis(c.Q);
+    return contact_apply(P, j.i, at, c, dichotomous_packed(c.Q), 0, 1, true, false);
+}
+
 __device__ __forceinline__ int2 contact_pairs_compacted(const Params &P, int np, float at, int chunk, int stride,
-                                                        int *q, int lane)
+                                                        QueuedPair *q, int lane)
 {
     const unsigned full = 0xffffffffu;
     int qn = 0;  // queued pairs (uniform over the warp)
     int2 counts = make_int2(0, 0);
+    int i = chunk * 32 + lane;
+    int2 next = i < np ? P.pair_v[i] : make_int2(0, 0);
     for (int base = chunk * 32; base < np; base += stride * 32) {
-        const int i = base + lane;
+        const int2 pv = next;
+        i = base + lane;
+        const int ahead = i + stride * 32;
+        if (ahead < np) next = P.pair_v[ahead];
         bool maybe = false;
         if (i < np) {
-            ContactPair c;
-            contact_load(P, i, c);
-            maybe = contact_may_touch(c.Q);
+            if (P.PB) {
+                maybe = boxes_may_touch(P, pv);
+            } else {
+                ContactPair c;
+                contact_load(P, i, c);
+                maybe = contact_may_touch(c.Q);
+            }
         }
         const unsigned m = __ballot_sync(full, maybe);
-        if (maybe) q[qn + __popc(m & ((1u << lane) - 1u))] = i;
+        if (maybe) q[qn + __popc(m & ((1u << lane) - 1u))] = QueuedPair{i, pv};
         qn += __popc(m);
         __syncwarp();
         if (qn >= 32) {
-            const int j = q[lane];
-            ContactPair c;
-            contact_load(P, j, c);
-            pill_pair_axis(c.Q);
-            const bool act = contact_apply(P, j, at, c, dichotomous(c.Q), 0, 1, true, false);
+            const bool act = queued_contact(P, q[lane], at);
             counts.x += 32;
             counts.y += __popc(__ballot_sync(full, act));
             __syncwarp();
@@ -1629,14 +1706,7 @@ __device__ __forceinline__ int2 contact_pairs_compacted(const Params &P, int np,
             __syncwarp();
         }
     }
-    bool act = false;
-    if (lane < qn) {
-        const int j = q[lane];
-        ContactPair c;
-        contact_load(P, j, c);
-        pill_pair_axis(c.Q);
-        act = contact_apply(P, j, at, c, dichotomous(c.Q), 0, 1, true, false);
-    }
+    const bool act = lane < qn && queued_contact(P, q[lane], at);
     counts.x += qn;
     counts.y += __popc(__ballot_sync(full, act));
     __syncwarp();

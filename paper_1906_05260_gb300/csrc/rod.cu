@@ -268,6 +268,7 @@ Params contact_path_params(const viper_scene *s)
     P.XW = (s->mode == VIPER_SOLVER_BATCHED && (s->flags & VIPER_FLAG_CONTACTS) && s->resident_nv == s->nv)
                ? s->xw
                : nullptr;
+    P.PB = P.XW ? s->pb : nullptr;
     return P;
 }
 

@@ -653,6 +653,84 @@ __device__ __forceinline__ float dichotomous(const PillPair &P)
     return 0.5f * (lo + hi);
 }
 
+// ---- both probes of a step at once: two floats in one 64-bit register, added,
+// multiplied and fused by the packed instructions (each half rounded as the
+// scalar one).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// a * b + c clamped to [0, 1] (NaN to 0), in one instruction
+__device__ __forceinline__ float fma_sat(float a, float b, float c)
+{
+    float r;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// dichotomous() with search_f of both probes packed: the same operations in
+// the same order, with the signs that the packed instructions cannot flip
+// moved into the coefficients (exact), 2 re as a product with 2 E0 and 2 E1
+// (exact), and the projection's clamp and its fixed case in one saturating
+// fused multiply-add.  Hence the same decisions, bit for bit.  Half the
+// arithmetic instructions of the scalar steps, which bound the contact pass.
+__device__ __forceinline__ float dichotomous_packed(const PillPair &P)
+{
+    const PillSearch S = pill_search(P);
+    const f32x2 A0 = pack2(S.A0, S.A0), A1 = pack2(S.A1, S.A1), minus = pack2(-1.f, -1.f);
+    const f32x2 R0 = pack2(S.R0, S.R0), R1 = pack2(S.R1, S.R1), R2 = pack2(S.R2, S.R2);
+    const f32x2 E0 = pack2(-2.f * S.E0, -2.f * S.E0), E1 = pack2(-2.f * S.E1, -2.f * S.E1), L2 = pack2(S.L2, S.L2);
+    const f32x2 ra = pack2(-S.ra1, -S.ra1), dra = pack2(-S.dra, -S.dra);
+    const f32x2 rb = pack2(-S.rb1, -S.rb1), drb = pack2(-S.drb, -S.drb), tn = pack2(-S.tn, -S.tn);
+    const bool fixed = S.fixed >= 0.f;
+    const float scale = fixed ? 0.f : S.inv_l, shift = fixed ? S.fixed : 0.f;
+    const f32x2 half = pack2(-0.5f, 0.5f);
+    float lo = 0.f, hi = 1.f;
+#pragma unroll 1
+    for (int it = 0; it < kDichoSteps; ++it) {
+        const float mid = 0.5f * (lo + hi), eps = 1e-3f * (hi - lo);
+        const f32x2 x = fma2(half, pack2(eps, eps), pack2(mid, mid));
+        const f32x2 a = fma2(x, A1, A0), rel = fma2(x, fma2(x, R2, R1), R0);
+        float h1, h2, t1, t2;
+        unpack2(fma2(mul2(a, minus), a, rel), h1, h2);
+        unpack2(fma2(pack2(sqrt_approx(fmaxf(h1, 0.f)), sqrt_approx(fmaxf(h2, 0.f))), tn, a), t1, t2);
+        const f32x2 t = pack2(fma_sat(t1, scale, shift), fma_sat(t2, scale, shift));
+        float d1, d2, f1, f2;
+        unpack2(fma2(t, fma2(t, L2, fma2(x, E1, E0)), rel), d1, d2);
+        const f32x2 dist = pack2(sqrt_approx(fmaxf(d1, 0.f)), sqrt_approx(fmaxf(d2, 0.f)));
+        unpack2(add2(add2(dist, fma2(x, dra, ra)), fma2(t, drb, rb)), f1, f2);
+        float x1, x2;
+        unpack2(x, x1, x2);
+        dicho_keep(lo, hi, x1, x2, f1 < f2);
+    }
+    return 0.5f * (lo + hi);
+}
+
 // The same search by one warp, four steps per round: the 2 + 4 + 8 + 16 probes
 // of the next four steps' possible brackets are evaluated at once (lane ->
 // depth j, node b = the earlier decisions of the round, side), then the four

@@ -104,6 +104,9 @@ struct Params {
     // world position and radius per vertex (x + rod origin, s rbar), written by the
     // shared-memory sweep before each contact pass and read by it; null: not used
     float4 *XW;
+    // with XW: per vertex the pill that starts there, as the contact pass's
+    // early-out reads it (pill_box): (midpoint, padded largest radius), (axis, its square)
+    float4 *PB;
     // contact-pass counters (null: not counted): candidate pairs, pairs searched by
     // the narrowphase (not excluded by the certified early-out), active constraints
     unsigned long long *contact_stats;
@@ -213,9 +216,9 @@ struct viper_scene {
     int *h_err = nullptr;
     int *d_herr = nullptr;  // its device address
     void *self_table = nullptr;  // one-scene table of the multi-scene kernels (graph path)
-    // world pack of the multi-kernel contact path (Params::XW), set only in the
+    // world and pill packs of the multi-kernel contact path (Params::XW, PB), set only in the
     // launch arguments of its sweeps and contact passes
-    float4 *xw = nullptr;
+    float4 *xw = nullptr, *pb = nullptr;
     // scratch for host-pointer skinning
     float4 *skin_buf = nullptr;
     size_t skin_cap = 0;
