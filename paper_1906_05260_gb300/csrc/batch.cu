@@ -481,6 +481,19 @@ __global__ void __launch_bounds__(256) batch_rod_first_kernel(BatchArgs A, int f
     rod_item_first(sb.P, local, finish_prev != 0, tau, sb.pills != 0, smem);
 }
 
+// Whether a scene's contact passes read world and pill packs (Params::XW, PB):
+// from the second sweep of a substep on, when the pair search found at least
+// two pairs per pill.  The sweep before such a pass writes them (48 bytes a
+// vertex); the same decision on both sides, from the pair count of the substep.
+// Scenes with few pairs do not pay for the packs; 45,000 pills of settled strands
+// (33 pairs a pill) take 7.7 ms a frame with this pass over up to four CTAs per SM,
+// 17.5 with 64 CTAs, scalar probes and no compaction.
+constexpr int kPackPairs = 2;
+__device__ __forceinline__ bool packs_used(const Params &P, bool first_sweep)
+{
+    return !first_sweep && P.XW && *P.npairs >= kPackPairs * P.ns;
+}
+
 // One colour sweep of every work item (contact path): FULL = false, or the
 // whole substep with all iterations (no contacts): FULL = true.
 template <bool FULL>
@@ -490,39 +503,42 @@ __global__ void __launch_bounds__(256, 2) batch_rod_kernel(BatchArgs A, int n_it
     extern __shared__ float4 smem[];
     int local, nblk;
     batch_enter(A, K_ROD, sb, local, nblk);
+    // read after rod_item's first barrier
+    if (!FULL && threadIdx.x == 0 && !packs_used(sb.P, first != 0)) sb.P.XW = nullptr;
     rod_item<FULL>(sb.P, local, n_iter, first != 0, apply != 0, tau, smem);
 }
 
-// Jacobi contact pass (Sec. 7.2): pairs, then half-plane vertices, over the scene's CTAs.
-__global__ void __launch_bounds__(kElemThreads) batch_contact_kernel(BatchArgs A)
+// Jacobi contact pass (Sec. 7.2) after the sweep `first`: pairs, then half-plane
+// vertices, over the scene's CTAs.
+__global__ void __launch_bounds__(kElemThreads, 4) batch_contact_kernel(BatchArgs A, int first)
 {
     __shared__ BatchScene sb;
+    __shared__ QueuedPair queue[kElemThreads / 32][64];
     int local, nblk;
     batch_enter(A, K_CONTACT, sb, local, nblk);
-    const Params &P = sb.P;
+    Params &P = sb.P;
+    if (threadIdx.x == 0 && !packs_used(P, first != 0)) {
+        P.XW = nullptr;
+        P.PB = nullptr;
+    }
     const int np_all = sb.pills ? *P.npairs : 0;
+    __syncthreads();
     const int np = min(np_all, P.max_pairs);
     if (local == 0 && threadIdx.x == 0 && np_all > P.max_pairs) atomicOr(P.err, ERR_OVERFLOW);
     const int nvp = P.n_planes > 0 ? P.nv : 0;
     const float at = P.contact_alpha * P.inv_h2;
     const int threads = nblk * blockDim.x;
+    const int lane = threadIdx.x & 31, warp = (local * blockDim.x + threadIdx.x) >> 5;
     if (!P.contact_threads && (long long)np * 16 <= threads) {
-        // few pairs (a scene's usual case, a few per cent of its pills): a warp
-        // per pair, at most two pairs per warp, the search's steps four at a
-        // time (three rounds against ten steps); then the vertices' half-plane
-        // constraints
-        const int lane = threadIdx.x & 31;
-        for (int i = (local * blockDim.x + threadIdx.x) >> 5; i < np; i += threads >> 5)
-            contact_pair_warp(P, i, at, lane);
-        for (int i = local * blockDim.x + threadIdx.x; i < nvp; i += threads) contact_planes(P, i, at);
-        return;
+        // few pairs (an animated scene's usual case, a few per cent of its pills): a
+        // warp per pair, at most two pairs per warp, the search's steps four at a
+        // time (three rounds against ten steps)
+        for (int i = warp; i < np; i += threads >> 5) contact_pair_warp(P, i, at, lane);
+    } else {
+        // a thread per pair, the pairs that may touch compacted per warp
+        contact_pairs_compacted(P, np, at, warp, threads >> 5, queue[threadIdx.x >> 5], lane);
     }
-    for (int i = local * blockDim.x + threadIdx.x; i < np + nvp; i += threads) {
-        if (i < np)
-            contact_pair(P, i, at);
-        else
-            contact_planes(P, i - np, at);
-    }
+    for (int i = local * blockDim.x + threadIdx.x; i < nvp; i += threads) contact_planes(P, i, at);
 }
 
 // Bundle shape matching after the substep's last contact pass (see
@@ -647,6 +663,8 @@ void launch(void (*kernel)(KArgs...), int grid, int block, int smem, cudaStream_
 // per warp (mode 2, a warp per 8 pills), which cuts the number of dependent
 // load chains by about 14.
 constexpr int kEmitPillsPerWarp = 8, kEmitPillsPerWarpSmall = 1, kEmitSmallGroup = 16384;
+// A contact CTA covers fewer pills in groups that do not fill the GPU (kEmitSmallGroup).
+constexpr int kContactPillsSmall = 64;
 constexpr int kMeshPerThread = 16;  // kLbsBatch vertices per round, 16 / kLbsBatch rounds
 
 size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -722,10 +740,14 @@ struct Shape {
 // scene's own target pose; the caller may point them elsewhere), and its
 // blocks per kernel kind.
 void fill_scene(BatchScene &b, int cnt[K_KINDS], viper_scene *s, const viper_batch_item &it, double h, bool cp,
-                int emit_ppw)
+                int emit_ppw, bool small)
 {
     memset(&b, 0, sizeof(b));
     b.P = s->P;
+    if ((s->flags & VIPER_FLAG_CONTACTS) && cp) {
+        b.P.XW = s->xw;
+        b.P.PB = s->pb;
+    }
     b.P.h = (float)h;
     b.P.inv_h = (float)(1.0 / h);
     b.P.inv_h2 = (float)(1.0 / (h * h));
@@ -751,7 +773,9 @@ void fill_scene(BatchScene &b, int cnt[K_KINDS], viper_scene *s, const viper_bat
     cnt[K_EMIT] = b.pills ? cdiv(ns, kEmitWarpsB * emit_ppw) : 0;  // about 0.4 emit_ppw work units per warp
     cnt[K_SCAN] = b.pills ? 1 : 0;
     cnt[K_ROD] = s->n_items;
-    cnt[K_CONTACT] = cp ? std::min(64, std::max(1, cdiv(ns + (s->n_planes > 0 ? nv : 0), kElemThreads))) : 0;
+    cnt[K_CONTACT] = cp ? std::min(4 * device_sm_count(),
+                                   std::max(1, cdiv(ns + (s->n_planes > 0 ? nv : 0), small ? kContactPillsSmall : kElemThreads)))
+                        : 0;
     cnt[K_END] = it.n_mesh > 0 ? std::max(1, cdiv(ns, kElemThreads)) : 1;
     cnt[K_MESH] = cdiv(it.n_mesh, kElemThreads * kMeshPerThread);
     cnt[K_BUNDLE] = cp ? cdiv(s->P.n_xs, kElemThreads / 32) : 0;
@@ -803,8 +827,8 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
     // the broadphase on a second branch beside the first sweep (not while profiling:
     // the per-class events bracket one stream)
     const bool forked = fork && fork->side && tot[K_PILL] > 0 && (!prof || prof->prof_class == PROF_NONE);
-    auto contact = [&]() {
-        go(PROF_CONTACT, [&] { launch(batch_contact_kernel, tot[K_CONTACT], kElemThreads, 0, st, A); });
+    auto contact = [&](int first) {
+        go(PROF_CONTACT, [&] { launch(batch_contact_kernel, tot[K_CONTACT], kElemThreads, 0, st, A, first); });
     };
     if (tot[K_WARM] > 0) go(PROF_ELEM, [&] { launch(batch_warm_kernel, tot[K_WARM], kElemThreads, 0, st, A); });
     if (cp && iterations > 0) {
@@ -825,10 +849,10 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
                 go(PROF_ROD, [&] { launch(batch_rod_first_kernel, tot[K_ROD], threads, smem, st, A, k > 0 ? 1 : 0, tau); });
                 broadphase(st);
             }
-            contact();
+            contact(1);
             for (int i = 1; i < iterations; ++i) {
                 go(PROF_ROD, [&] { launch(batch_rod_kernel<false>, tot[K_ROD], threads, smem, st, A, 1, 0, 1, tau); });
-                contact();
+                contact(0);
             }
             if (tot[K_BUNDLE] > 0)
                 go(PROF_ELEM, [&] { launch(batch_bundle_kernel, tot[K_BUNDLE], kElemThreads, 0, st, A); });
@@ -890,7 +914,7 @@ int run_group(viper_batch *B, const viper_batch_item *items, const std::vector<i
         viper_scene *s = it.scene;
         BatchScene &b = hs[k];
         int cnt[K_KINDS];
-        fill_scene(b, cnt, s, it, h, cp, emit_ppw);
+        fill_scene(b, cnt, s, it, h, cp, emit_ppw, small_group);
         if (it.bone_quat && s->n_bones > 0) {  // this frame's target pose, from the call's table
             memcpy(hbq + bcur, it.bone_quat, sizeof(float4) * s->n_bones);
             memcpy(hbt + 3 * bcur, it.bone_trans, sizeof(float) * 3 * s->n_bones);
@@ -905,7 +929,7 @@ int run_group(viper_batch *B, const viper_batch_item *items, const std::vector<i
     // a warp per contact pair shortens one scene's chain but multiplies the
     // lanes' work; once the scenes' contact passes fill the GPU, throughput
     // decides: one thread per pair
-    if (sh.tot[K_CONTACT] > device_sm_count())
+    if (!small_group && sh.tot[K_CONTACT] > device_sm_count())
         for (int k = 0; k < n; ++k) hs[k].P.contact_threads = 1;
 
     cudaStream_t st = B->stream;
@@ -947,7 +971,7 @@ int self_batch_capture(viper_scene *s, float dt, int substeps, int iterations, c
     int cnt[K_KINDS];
     const bool small_group = s->ns <= kEmitSmallGroup;
     const int emit_ppw = small_group ? kEmitPillsPerWarpSmall : kEmitPillsPerWarp;
-    fill_scene(*b, cnt, s, it, (double)dt / substeps, cp, emit_ppw);  // bones: the scene's own target pose
+    fill_scene(*b, cnt, s, it, (double)dt / substeps, cp, emit_ppw, small_group);  // bones: the scene's own target pose
     Shape sh;
     shape_add(sh, s, cp);
     sh.emit_mode = small_group ? 1 : 2;
