@@ -30,7 +30,7 @@
 
 namespace viper {
 
-enum BatchKind : int { K_ELEM = 0, K_PILL, K_EMIT, K_SCAN, K_ROD, K_CONTACT, K_END, K_MESH, K_BUNDLE, K_WARM, K_KINDS };
+enum BatchKind : int { K_ELEM = 0, K_PILL, K_EMIT, K_SCAN, K_GRID, K_ROD, K_CONTACT, K_END, K_MESH, K_BUNDLE, K_WARM, K_KINDS };
 
 // One scene of a batched frame, as the device sees it.
 struct BatchScene {
@@ -60,7 +60,7 @@ constexpr int kElemThreads = 256, kEmitWarpsB = 8, kScanThreadsB = 1024, kScanPe
 // staged in shared memory; local = block index within the scene, nblk = its block count.
 // Kernels are launched with programmatic dependent launch (see pdl_wait): this
 // prologue overlaps the predecessor kernel.
-__device__ __forceinline__ void batch_enter(const BatchArgs &A, int kind, BatchScene &sb, int &local, int &nblk)
+__device__ __forceinline__ void batch_scene(const BatchArgs &A, int kind, BatchScene &sb, int &local, int &nblk)
 {
     __shared__ int s_lo, s_hi;
     const int *o = A.off + kind * (A.n + 1);
@@ -81,6 +81,11 @@ __device__ __forceinline__ void batch_enter(const BatchArgs &A, int kind, BatchS
     __syncthreads();
     local = b - s_lo;
     nblk = s_hi - s_lo;
+}
+
+__device__ __forceinline__ void batch_enter(const BatchArgs &A, int kind, BatchScene &sb, int &local, int &nblk)
+{
+    batch_scene(A, kind, sb, local, nblk);
     // Everything above reads only the call's table, uploaded before the first
     // kernel of the call; the scene state is read after the predecessor kernel
     // has finished.  The successor is released once every CTA got here.
@@ -179,295 +184,369 @@ __global__ void __launch_bounds__(kElemThreads) batch_scatter_kernel(BatchArgs A
     }
 }
 
-// Candidate pairs, one warp per work unit.  With a grid from batch_grid_kernel:
-// mode 1, a 32-pill chunk against one neighbour list (see emit_chunk), for groups
-// of few pills; mode 2, a chunk against all its neighbour lists (see
-// emit_chunk_all), for many.  Mode 0 (grid from the multi-kernel build): a cell
-// against one neighbour cell (see emit_cell).
-__global__ void __launch_bounds__(32 * kEmitWarpsB) batch_emit_kernel(BatchArgs A, int mode)
+// Candidate pairs, L lanes per pill (see emit_pills; no oversized pills here:
+// the cell is sized for the largest).
+template <int L>
+__global__ void __launch_bounds__(32 * kEmitWarpsB) batch_emit_kernel(BatchArgs A)
 {
     __shared__ BatchScene sb;
+    __shared__ int buf[kEmitWarpsB][kEmitBuf];
     int local, nblk;
     batch_enter(A, K_EMIT, sb, local, nblk);
     const Params &P = sb.P;
     const Grid G = *P.grid;
-    const int n_chunks = mode > 0 ? *P.n_chunks : 0;  // loaded beside the grid, not after the test
     if (G.pad) return;  // no valid grid: no candidates (uniform over the CTA)
     const int wib = threadIdx.x >> 5;
-    const int cells = grid_cells(P.grid, P.table);
-    const int *cs = P.cell_start;
-    auto start = [cs](int c) { return cs[c]; };
-    __shared__ float4 s_cand[kEmitWarpsB][32];  // per warp: the neighbour block being tested
-    __shared__ int s_cgrp[kEmitWarpsB][32], s_cid[kEmitWarpsB][32];
-    if (mode == 2) {  // a chunk with all its neighbour lists per warp
-        const int n = n_chunks;
-        for (int q = local * kEmitWarpsB + wib; q < n; q += nblk * kEmitWarpsB)
-            emit_chunk_all<4>(P, G, q, start, s_cand[wib], s_cgrp[wib], s_cid[wib]);
-    } else if (mode == 1) {  // a chunk with one neighbour list per warp
-        const int n = kEmitUnits * n_chunks;
-        for (int u = local * kEmitWarpsB + wib; u < n; u += nblk * kEmitWarpsB)
-            emit_chunk<4>(P, G, u, start, s_cand[wib], s_cgrp[wib], s_cid[wib]);
-    } else {
-        for (int u = local * kEmitWarpsB + wib; u < kEmitUnits * cells; u += nblk * kEmitWarpsB)
-            emit_cell<4>(P, G, u, start);
-    }
+    const int n = P.cell_start[grid_cells(&G, P.table)];  // pills in the cells
+    emit_pills<L>(P, G, 0xffffffffu, n, local * kEmitWarpsB + wib, nblk * kEmitWarpsB, buf[wib], threadIdx.x & 31);
 }
 
-// One scene's broadphase grid by one CTA: bounding spheres and their bounds,
-// the grid, cell counts, the exclusive cell scan into cell_start (and the
-// list of 32-pill chunks per cell, chunk_of), and the scatter into cell order
-// with the sphere / group copies.
-//
-// Small scenes (at most kGridSmemVerts vertices and kGridSmemCells cells) run
-// from shared memory: the spheres are built per vertex slot (vertex v starts a
-// pill when vtx_seg[v + 1] = vtx_seg[v] + 1, so all loads of a slot are
-// independent), cell counts and offsets live in shared memory, the scan runs
-// warp-strided over consecutive cells (conflict-free, coalesced stores), and
-// the scatter goes through a shared permutation so that the cell-order arrays
-// are written with coalesced stores.  Larger scenes take the general path:
-// spheres and cells in global memory, counts in shared memory when the grid
-// spans at most kGridSmemCells cells, else in cell_count.
-constexpr int kGridThreads = 512, kGridSmemCells = 8192, kGridMaxPills = 1 << 16, kGridSmemVerts = 8192;
-constexpr int kGridSmemBytes = 4 * kGridSmemCells + (16 + 4 + 4) * kGridSmemVerts;  // 224 KB
-
-// Warp-strided exclusive scan of cnt[0, cells) into cnt (as each cell's fill
-// position) and cell_start, with the 32-pill chunks of every cell listed in
-// chunk_of.  Warp w owns cells [w m 32, (w + 1) m 32), m = ceil(cells / (32 W)).
-// cnt is shared memory, or cell_count (`global`: written by atomics, read from L2).
-__device__ __forceinline__ void grid_scan(const Params &P, int *cnt, int cells, int *ws, bool global)
+// ---------------------------------------------------------------- one scene's grid by one cluster
+__device__ __forceinline__ unsigned cluster_rank()
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int m = (cells + 32 * nw - 1) / (32 * nw);
-    const int c0 = w * m * 32;
-    int s = 0, cs = 0;
-    for (int j = 0; j < m; ++j) {
-        const int c = c0 + 32 * j + lane;
-        const int v = c < cells ? (global ? __ldcg(cnt + c) : cnt[c]) : 0;
-        s += v;
-        cs += (v + 31) >> 5;
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ unsigned cluster_ctas()
+{
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+// Every thread of the cluster calls both; they order shared and global memory between its CTAs.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync()
+{
+    cluster_arrive();
+    cluster_wait();
+}
+// Address of shared variable p in CTA `rank` of the cluster.
+__device__ __forceinline__ unsigned in_cta(const void *p, unsigned rank)
+{
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;"
+        : "=r"(r)
+        : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_store(unsigned addr, unsigned v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ int cluster_load(unsigned addr)
+{
+    int v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ int cluster_add(unsigned addr, int v)
+{
+    int r;
+    asm volatile("atom.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(r) : "r"(addr), "r"(v) : "memory");
+    return r;
+}
+
+// One scene's broadphase grid by one cluster of CTAs: bounding spheres and their
+// bounds, the grid, cell counts, the exclusive cell scan into cell_start, and
+// the scatter into cell order with the sphere / group copies.
+//
+// Pills that can touch no pill of another group are left out first (scenes of up
+// to kGridGroupsMax groups): a group's box, enlarged well above the rounding of
+// spheres_overlap, bounds its pills' spheres; where two groups' boxes meet, a
+// pill of either can only touch the other's inside the meeting of the boxes; and
+// a pill stays if it reaches the box around its group's meetings.  A rig's
+// muscles lie side by side: of 6,910 pills 24 stay, where the cells (as wide as
+// the largest pill, nine times the smallest) held 180 candidates a pill, nearly
+// all of the pill's own muscle.
+//
+// The build is a chain of dependent phases, too short for a launch each and too
+// long for one CTA (10,080 pills: 38.5 us by one CTA of 512 threads, 18.4 by eight).
+// The cluster splits the pills into slices and the cells into ranges of 2^sh,
+// one of each per CTA, all in shared memory: spheres and the pills' cells in
+// their slice, counts and starts in the range's owner.  Counting a pill returns
+// its place within its cell, so that the scatter needs no second pass of atomics.
+// The CTAs meet five times (boxes, bounds, counts, range totals, end).
+// Dynamic shared memory: slice_cap spheres, cells (first the pills' vertices) and
+// places (first their groups), cells_cap cell counts (the table's share of a CTA, a
+// power of two), and per group this CTA's and the scene's box (6 words each).
+constexpr int kGridThreads = 512, kGridClusterMax = 8, kGridCellsMax = 16384, kGridSliceMax = 6144;
+constexpr int kGridMaxPills = kGridClusterMax * kGridSliceMax;  // 49,152: table of 131,072 cells = 8 x kGridCellsMax
+constexpr int kGridGroupsMax = 512;
+inline int grid_smem_bytes(int cells_cap, int slice_cap, int groups_cap)
+{
+    return (16 + 4 + 4) * slice_cap + 4 * cells_cap + 48 * groups_cap;
+}
+
+// Half-width of the box of sphere sp in the cull: its radius and a margin far above
+// the rounding of the box and of spheres_overlap.
+__device__ __forceinline__ float cull_reach(float4 sp)
+{
+    return 1.0078125f * fabsf(sp.w) + 1e-6f * (fabsf(sp.x) + fabsf(sp.y) + fabsf(sp.z));
+}
+
+__device__ __forceinline__ void cluster_max(unsigned addr, unsigned v)
+{
+    asm volatile("red.shared::cluster.max.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// Sphere sp of a pill of group grp into the box table (six words as in
+// merge_bounds_to); the lanes `act` call it together, one addition per group.
+__device__ __forceinline__ void box_add(unsigned *box, unsigned act, int grp, float4 sp)
+{
+    const unsigned peers = __match_any_sync(act, grp);
+    const float r = cull_reach(sp);
+    const bool in = isfinite(sp.x + sp.y + sp.z + r);  // no pair has a sphere that is not
+    const float c[3] = {sp.x, sp.y, sp.z};
+    unsigned w[6];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        w[k] = __reduce_max_sync(peers, in ? ord_enc(r - c[k]) : 0u);
+        w[3 + k] = __reduce_max_sync(peers, in ? ord_enc(c[k] + r) : 0u);
+    }
+    if ((threadIdx.x & 31) == __ffs(peers) - 1)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) atomicMax(box + 6 * grp + k, w[k]);
+}
+
+// The box around group a's meetings with the other groups' boxes, by one warp,
+// written to hot (as floats: low, high; empty: low above high).
+__device__ __forceinline__ void hot_box(const unsigned *box, int groups, int a, float *hot, int lane)
+{
+    float lo[3], hi[3], hl[3] = {INFINITY, INFINITY, INFINITY}, hh[3] = {-INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        lo[k] = -ord_dec(box[6 * a + k]);
+        hi[k] = ord_dec(box[6 * a + 3 + k]);
+    }
+    for (int b = lane; b < groups; b += 32) {
+        if (b == a || box[6 * b] == 0u) continue;
+        float l[3], h[3];
+        bool meet = true;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            l[k] = fmaxf(lo[k], -ord_dec(box[6 * b + k]));
+            h[k] = fminf(hi[k], ord_dec(box[6 * b + 3 + k]));
+            meet = meet && l[k] <= h[k];
+        }
+        if (meet)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                hl[k] = fminf(hl[k], l[k]);
+                hh[k] = fmaxf(hh[k], h[k]);
+            }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        cs += __shfl_xor_sync(0xffffffffu, cs, o);
-    }
-    if (lane == 0) {
-        ws[w] = s;
-        ws[16 + w] = cs;
-    }
-    __syncthreads();
-    if (w == 0) {  // exclusive prefix of the warp totals (at most 16 warps)
-        const int a = lane < nw ? ws[lane] : 0, b = lane < nw ? ws[16 + lane] : 0;
-        const int ia = warp_incl_scan(a), ib = warp_incl_scan(b);
-        __syncwarp();
-        if (lane < nw) {
-            ws[lane] = ia - a;
-            ws[16 + lane] = ib - b;
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            hl[k] = fminf(hl[k], __shfl_xor_sync(0xffffffffu, hl[k], o));
+            hh[k] = fmaxf(hh[k], __shfl_xor_sync(0xffffffffu, hh[k], o));
         }
-        if (lane == nw - 1) {
-            P.cell_start[cells] = ia;
-            *P.n_chunks = ib;
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            hot[k] = hl[k];
+            hot[3 + k] = hh[k];
         }
-    }
-    __syncthreads();
-    int off = ws[w], coff = ws[16 + w];
-    int4 *chunk_of = P.chunk_of;
-    int *cell_start = P.cell_start;
-    for (int j = 0; j < m; ++j) {
-        const int c = c0 + 32 * j + lane;
-        const int v = c < cells ? (global ? __ldcg(cnt + c) : cnt[c]) : 0, nch = (v + 31) >> 5;
-        const int iv = warp_incl_scan(v), ic = warp_incl_scan(nch);
-        if (c < cells) {
-            const int o = off + iv - v, oc = coff + ic - nch;
-            cell_start[c] = o;
-            cnt[c] = o;
-            for (int h = 0; h < nch; ++h) chunk_of[oc + h] = make_int4(c, o + 32 * h, min(o + 32 * h + 32, o + v), o + v);
-        }
-        off += __shfl_sync(0xffffffffu, iv, 31);
-        coff += __shfl_sync(0xffffffffu, ic, 31);
-    }
 }
 
-__global__ void __launch_bounds__(kGridThreads) batch_grid_kernel(BatchArgs A)
+__global__ void __launch_bounds__(kGridThreads, 2)
+    batch_grid_kernel(BatchArgs A, int cells_cap, int slice_cap, int groups_cap)
 {
     __shared__ BatchScene sb;
-    __shared__ unsigned int s_bounds[8];
+    __shared__ unsigned int s_bounds[8], s_kept[8];     // of all pills, of those that stay
+    __shared__ unsigned int s_all[kGridClusterMax][8];  // the CTAs' bounds
+    __shared__ unsigned int s_all_kept[kGridClusterMax][8];
+    __shared__ int s_tot[kGridClusterMax];              // the ranges' totals
     __shared__ int ws[33];
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    int *s_cells = reinterpret_cast<int *>(s_dyn);
+    float4 *s_sph = reinterpret_cast<float4 *>(s_dyn);
+    int *s_cell = reinterpret_cast<int *>(s_sph + slice_cap);
+    int *s_place = s_cell + slice_cap;
+    int *s_count = s_place + slice_cap;
+    unsigned *s_own = reinterpret_cast<unsigned *>(s_count + cells_cap), *s_box = s_own + 6 * groups_cap;
     int local, nblk;
-    batch_enter(A, K_SCAN, sb, local, nblk);
+    batch_scene(A, K_GRID, sb, local, nblk);
     const Params &P = sb.P;
-    const int t = threadIdx.x, bd = blockDim.x, ns = P.ns, nv = P.nv;
-    if (t < 8) s_bounds[t] = 0u;
+    const int t = threadIdx.x, bd = blockDim.x, ns = P.ns;
+    const unsigned rank = cluster_rank(), ctas = cluster_ctas();
+    const int per = (ns + (int)ctas - 1) / (int)ctas;
+    const int g0 = min((int)rank * per, ns), n = min(per, ns - g0);  // this CTA's pills [g0, g0 + n)
+    // before the predecessor has finished: what does not depend on the state
+    const int groups = P.n_groups <= groups_cap ? P.n_groups : 0;  // 0: every pill stays
+    if (t < 8) s_bounds[t] = s_kept[t] = 0u;
+    for (int c = t; c < cells_cap; c += bd) s_count[c] = 0;
+    for (int c = t; c < 6 * groups; c += bd) s_own[c] = s_box[c] = 0u;
+    for (int i = t; i < n; i += bd) {
+        s_cell[i] = P.seg_v0[g0 + i];
+        s_place[i] = P.seg_group[g0 + i];
+    }
     __syncthreads();
+    cluster_arrive();
+    pdl_wait();
+    pdl_trigger();
+
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY}, mr = 0.f;
-    const bool small = nv <= kGridSmemVerts;  // uniform over the CTA
-    float4 *s_sph = reinterpret_cast<float4 *>(s_dyn + 4 * kGridSmemCells);
-    int *s_pill = reinterpret_cast<int *>(s_dyn + 4 * kGridSmemCells + 16 * kGridSmemVerts);
-    int *s_perm = reinterpret_cast<int *>(s_dyn + 4 * kGridSmemCells + 20 * kGridSmemVerts);
-    if (small) {
-        const int *vtx_seg = P.vtx_seg;
+    {
         const float4 *xp = P.Xpred;
         const float *rbar = P.bp_rbar;
         const size_t rs = (size_t)P.bp_rbar_stride;
-        for (int base = 0; base < nv; base += 8 * bd) {
-            int ga[8], gb[8];
-            float4 xa[8], xb[8];
-            float ra[8], rb[8];
+        for (int base = 0; base < n; base += 4 * bd) {  // 4 pills per thread and batch, loads issued together
+            float4 xa[4], xb[4];
+            float ra[4], rb[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int v = base + k * bd + t;
-                const bool ok = v + 1 < nv;
-                ga[k] = ok ? vtx_seg[v] : 0;
-                gb[k] = ok ? vtx_seg[v + 1] : 0;
-                xa[k] = ok ? xp[v] : make_float4(0.f, 0.f, 0.f, 0.f);
-                xb[k] = ok ? xp[v + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
-                ra[k] = ok ? rbar[(size_t)v * rs] : 0.f;
-                rb[k] = ok ? rbar[(size_t)(v + 1) * rs] : 0.f;
+            for (int k = 0; k < 4; ++k) {
+                const int i = base + k * bd + t;
+                const size_t a = i < n ? s_cell[i] : 0;
+                xa[k] = xp[a];
+                xb[k] = xp[a + 1];
+                ra[k] = rbar[a * rs];
+                rb[k] = rbar[(a + 1) * rs];
             }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int v = base + k * bd + t;
-                if (v >= nv) continue;
-                const bool pill = v + 1 < nv && gb[k] == ga[k] + 1;  // v and v + 1 on one rod
-                s_pill[v] = pill ? ga[k] : -1;
-                if (pill) {
-                    const float4 sp = pill_sphere(xa[k], ra[k], xb[k], rb[k]);
-                    s_sph[v] = sp;
-                    mn[0] = fminf(mn[0], sp.x); mn[1] = fminf(mn[1], sp.y); mn[2] = fminf(mn[2], sp.z);
-                    mx[0] = fmaxf(mx[0], sp.x); mx[1] = fmaxf(mx[1], sp.y); mx[2] = fmaxf(mx[2], sp.z);
-                    mr = fmaxf(mr, sp.w);
-                }
-            }
-        }
-    } else {
-        for (int g0 = 0; g0 < ns; g0 += 8 * bd) {  // 8 pills per thread and batch, loads issued together
-            int av[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int g = g0 + k * bd + t;
-                av[k] = g < ns ? P.seg_v0[g] : -1;
-            }
-            float4 sp[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int a = av[k] < 0 ? 0 : av[k];
-                sp[k] = pill_sphere(P.Xpred[a], P.bp_rbar[(size_t)a * P.bp_rbar_stride], P.Xpred[a + 1],
-                                    P.bp_rbar[(size_t)(a + 1) * P.bp_rbar_stride]);
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                if (av[k] < 0) continue;
-                P.spheres[g0 + k * bd + t] = sp[k];
-                mn[0] = fminf(mn[0], sp[k].x); mn[1] = fminf(mn[1], sp[k].y); mn[2] = fminf(mn[2], sp[k].z);
-                mx[0] = fmaxf(mx[0], sp[k].x); mx[1] = fmaxf(mx[1], sp[k].y); mx[2] = fmaxf(mx[2], sp[k].z);
-                mr = fmaxf(mr, sp[k].w);
+            for (int k = 0; k < 4; ++k) {
+                const int i = base + k * bd + t;
+                const unsigned act = __ballot_sync(0xffffffffu, i < n);
+                if (i >= n) continue;
+                const float4 sp = pill_sphere(xa[k], ra[k], xb[k], rb[k]);
+                s_sph[i] = sp;
+                if (groups) box_add(s_own, act, s_place[i], sp);
+                mn[0] = fminf(mn[0], sp.x); mn[1] = fminf(mn[1], sp.y); mn[2] = fminf(mn[2], sp.z);
+                mx[0] = fmaxf(mx[0], sp.x); mx[1] = fmaxf(mx[1], sp.y); mx[2] = fmaxf(mx[2], sp.z);
+                mr = fmaxf(mr, sp.w);
             }
         }
     }
     merge_bounds_to(s_bounds, mn, mx, mr);
     __syncthreads();
+    cluster_wait();  // every CTA of the cluster has started
+    for (int k = t; k < 8 * (int)ctas; k += bd) cluster_store(in_cta(&s_all[rank][k & 7], k >> 3), s_bounds[k & 7]);
+    for (int k = t; k < 6 * groups; k += bd)
+        if (s_own[k])
+            for (unsigned r = 0; r < ctas; ++r) cluster_max(in_cta(s_box + k, r), s_own[k]);
+    cluster_sync();  // bounds and boxes exchanged
+    if (t < 8) {
+        unsigned int m = 0u;
+        for (unsigned r = 0; r < ctas; ++r) m = max(m, s_all[r][t]);
+        s_bounds[t] = m;
+    }
+    __syncthreads();
     bool ok;
-    const Grid G = make_grid_from(s_bounds, P.table, ok);
+    Grid G;
+    if (groups) {
+        // the groups of this CTA's pills: their meetings with the others, then the pills that reach them
+        const int lane = t & 31;
+        for (int a = t >> 5; a < groups; a += bd >> 5)
+            if (s_own[6 * a]) hot_box(s_box, groups, a, reinterpret_cast<float *>(s_own + 6 * a), lane);
+        __syncthreads();
+        float kn[3] = {INFINITY, INFINITY, INFINITY}, kx[3] = {-INFINITY, -INFINITY, -INFINITY}, kr = 0.f;
+        for (int i = t; i < n; i += bd) {
+            const float4 sp = s_sph[i];
+            const float r = cull_reach(sp), *hot = reinterpret_cast<const float *>(s_own + 6 * s_place[i]);
+            const bool stays = sp.x - r <= hot[3] && sp.y - r <= hot[4] && sp.z - r <= hot[5] && sp.x + r >= hot[0] &&
+                               sp.y + r >= hot[1] && sp.z + r >= hot[2];
+            s_cell[i] = stays ? 0 : -1;
+            if (!stays) continue;
+            kn[0] = fminf(kn[0], sp.x); kn[1] = fminf(kn[1], sp.y); kn[2] = fminf(kn[2], sp.z);
+            kx[0] = fmaxf(kx[0], sp.x); kx[1] = fmaxf(kx[1], sp.y); kx[2] = fmaxf(kx[2], sp.z);
+            kr = fmaxf(kr, fabsf(sp.w));
+        }
+        __syncwarp();
+        merge_bounds_to(s_kept, kn, kx, kr);
+        __syncthreads();
+        for (int k = t; k < 8 * (int)ctas; k += bd)
+            cluster_store(in_cta(&s_all_kept[rank][k & 7], k >> 3), s_kept[k & 7]);
+        cluster_sync();
+        if (t < 8) {
+            unsigned int m = 0u;
+            for (unsigned r = 0; r < ctas; ++r) m = max(m, s_all_kept[r][t]);
+            s_kept[t] = m;
+        }
+        __syncthreads();
+        make_grid_from(s_bounds, P.table, ok);  // ok: of all pills, as without the cull
+        bool some;
+        G = make_grid_from(s_kept, P.table, some);
+        if (!ok) G.pad = 1;
+    } else {
+        G = make_grid_from(s_bounds, P.table, ok);
+    }
     const int cells = (int)min((long long)G.dim[0] * G.dim[1] * G.dim[2], (long long)P.table);
-    const bool in_smem = cells <= kGridSmemCells;
-    // counts in s_cells, or in cell_count (zero between substeps) for larger grids
-    if (in_smem)
-        for (int c = t; c < cells; c += bd) s_cells[c] = 0;
-    if (t == 0) {
+    int sh = 5;  // cells per CTA: 2^sh, at most cells_cap (the table holds at most cells_cap x ctas cells)
+    while (((int)ctas << sh) < cells) ++sh;
+    if (rank == 0 && t == 0) {
         *P.grid = G;
         *P.npairs = 0;
         if (!ok) atomicOr(P.err, ERR_NONFINITE);
     }
+    for (int i = t; i < n; i += bd) {
+        if (groups && s_cell[i] < 0) continue;
+        const int cell = bp_cell(G, s_sph[i]);
+        s_cell[i] = cell;
+        s_place[i] = cluster_add(in_cta(s_count + (cell & ((1 << sh) - 1)), cell >> sh), 1);
+    }
+    cluster_sync();  // counts complete
+    // exclusive scan of this CTA's cells, warp-strided over consecutive cells
+    const int lane = t & 31, w = t >> 5, nw = bd >> 5;
+    const int own = max(0, min(1 << sh, cells - ((int)rank << sh)));
+    const int m = (own + 32 * nw - 1) / (32 * nw), c0 = w * m * 32;
+    int sum = 0;
+    for (int j = 0; j < m; ++j) {
+        const int c = c0 + 32 * j + lane;
+        sum += c < own ? s_count[c] : 0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) ws[w] = sum;
     __syncthreads();
-    if (small && in_smem) {
-        for (int v = t; v < nv; v += bd)
-            if (s_pill[v] >= 0) atomicAdd(s_cells + bp_cell(G, s_sph[v]), 1);
-        __syncthreads();
-        grid_scan(P, s_cells, cells, ws, false);
-        __syncthreads();
-        // cell-order slot of every pill into the shared permutation, then the
-        // cell-order arrays with coalesced stores
-        for (int v = t; v < nv; v += bd)
-            if (s_pill[v] >= 0) s_perm[atomicAdd(s_cells + bp_cell(G, s_sph[v]), 1)] = v;
-        __syncthreads();
+    if (w == 0) {  // exclusive prefix of the warp totals (at most 16 warps)
+        const int a = lane < nw ? ws[lane] : 0;
+        const int ia = warp_incl_scan(a);
+        __syncwarp();
+        if (lane < nw) ws[lane] = ia - a;
+        const int total = __shfl_sync(0xffffffffu, ia, 31);
+        if (lane < (int)ctas) cluster_store(in_cta(s_tot + rank, lane), (unsigned)total);
+    }
+    __syncthreads();
+    int off = ws[w];
+    for (int j = 0; j < m; ++j) {
+        const int c = c0 + 32 * j + lane;
+        const int v = c < own ? s_count[c] : 0;
+        const int iv = warp_incl_scan(v);
+        if (c < own) s_count[c] = off + iv - v;
+        off += __shfl_sync(0xffffffffu, iv, 31);
+    }
+    cluster_sync();  // the ranges' starts and totals
+    if (t == 0) {  // totals to the ranges' first entries
+        int a = 0;
+        for (unsigned r = 0; r < ctas; ++r) {
+            const int v = s_tot[r];
+            s_tot[r] = a;
+            a += v;
+        }
+        if (rank == 0) P.cell_start[cells] = a;
+    }
+    __syncthreads();
+    {
         const int *seg_group = P.seg_group;
         int *cell_pills = P.cell_pills, *cell_grp = P.cell_grp;
         float4 *cell_sph = P.cell_sph;
-        for (int q0 = 0; q0 < ns; q0 += 8 * bd) {
-            int vq[8], gq[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int q = q0 + k * bd + t;
-                vq[k] = q < ns ? s_perm[q] : 0;
-                gq[k] = q < ns ? seg_group[s_pill[vq[k]]] : 0;
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int q = q0 + k * bd + t;
-                if (q < ns) {
-                    cell_pills[q] = s_pill[vq[k]];
-                    cell_sph[q] = s_sph[vq[k]];
-                    cell_grp[q] = gq[k];
-                }
-            }
-        }
-        return;
-    }
-    // general path
-    if (small) {  // spheres were built in shared memory: hand them to the global arrays
-        for (int v = t; v < nv; v += bd)
-            if (s_pill[v] >= 0) P.spheres[s_pill[v]] = s_sph[v];
-        __syncthreads();
-    }
-    for (int g0 = 0; g0 < ns; g0 += 8 * bd) {
-        float4 sp[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int g = g0 + k * bd + t;
-            sp[k] = g < ns ? P.spheres[g] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int g = g0 + k * bd + t;
-            if (g >= ns) continue;
-            const int cell = bp_cell(G, sp[k]);
-            P.cell_of[g] = cell;
-            if (in_smem)
-                atomicAdd(s_cells + cell, 1);
-            else
-                atomicAdd(P.cell_count + cell, 1);
+        for (int i = t; i < n; i += bd) {
+            const int cell = s_cell[i], r = cell >> sh;
+            if (cell < 0) continue;
+            const int pos = s_tot[r] + cluster_load(in_cta(s_count + (cell & ((1 << sh) - 1)), r)) + s_place[i];
+            cell_pills[pos] = g0 + i;
+            cell_sph[pos] = s_sph[i];
+            cell_grp[pos] = seg_group[g0 + i];
         }
     }
-    __syncthreads();
-    grid_scan(P, in_smem ? s_cells : P.cell_count, cells, ws, !in_smem);
-    __syncthreads();
-    for (int g0 = 0; g0 < ns; g0 += 8 * bd) {
-        int cq[8], gq[8];
-        float4 sp[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int g = g0 + k * bd + t;
-            const bool ok = g < ns;
-            cq[k] = ok ? P.cell_of[g] : 0;
-            gq[k] = ok ? P.seg_group[g] : 0;
-            sp[k] = ok ? P.spheres[g] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int g = g0 + k * bd + t;
-            if (g >= ns) continue;
-            const int pos = in_smem ? atomicAdd(s_cells + cq[k], 1) : atomicAdd(P.cell_count + cq[k], 1);
-            P.cell_pills[pos] = g;
-            P.cell_sph[pos] = sp[k];
-            P.cell_grp[pos] = gq[k];
-        }
+    {
+        int *cell_start = P.cell_start;
+        const int base = s_tot[rank], first = (int)rank << sh;
+        for (int c = t; c < own; c += bd) cell_start[first + c] = base + s_count[c];
     }
-    if (!in_smem) {  // return cell_count to zero for the next substep
-        __syncthreads();
-        for (int c = t; c < cells; c += bd) P.cell_count[c] = 0;
-    }
+    cluster_sync();  // the others have read this CTA's starts
 }
 
 // First sweep of a substep with the previous substep's velocity update and
@@ -641,30 +720,48 @@ namespace {
 
 // Launch with programmatic stream serialisation (the kernel's prologue may
 // overlap its predecessor; see batch_enter).
+// launch_clusters: in thread-block clusters of `ctas`.
 template <typename... KArgs, typename... Args>
-void launch(void (*kernel)(KArgs...), int grid, int block, int smem, cudaStream_t st, Args... args)
+void launch_clusters(void (*kernel)(KArgs...), int grid, int ctas, int block, int smem, cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = ctas;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = ctas > 1 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Pair search shape: a scene has about ns / 32 + (occupied cells) chunks of 14
-// units.  Groups of few pills run one unit per warp (mode 1, a warp per pill,
-// so the units' dependent loads run side by side); large groups run one chunk
-// per warp (mode 2, a warp per 8 pills), which cuts the number of dependent
-// load chains by about 14.
-constexpr int kEmitPillsPerWarp = 8, kEmitPillsPerWarpSmall = 1, kEmitSmallGroup = 16384;
-// A contact CTA covers fewer pills in groups that do not fill the GPU (kEmitSmallGroup).
-constexpr int kContactPillsSmall = 64;
+template <typename... KArgs, typename... Args>
+void launch(void (*kernel)(KArgs...), int grid, int block, int smem, cudaStream_t st, Args... args)
+{
+    launch_clusters(kernel, grid, 1, block, smem, st, args...);
+}
+
+// CTAs of the cluster that builds a scene's grid: eight where that fills no more
+// than the GPU's two CTAs per SM, fewer for many scenes, but enough for the
+// largest scene's cells and pills (kGridCellsMax, kGridSliceMax per CTA).
+int grid_cluster(int scenes, int max_ns, int max_table)
+{
+    int c = scenes * kGridClusterMax <= 2 * device_sm_count() ? kGridClusterMax : scenes <= device_sm_count() ? 4 : 2;
+    while (c < kGridClusterMax && (max_table > c * kGridCellsMax || max_ns > c * kGridSliceMax)) c *= 2;
+    return c;
+}
+
+// Groups of few pills do not fill the GPU with a thread per pill: several lanes
+// search a pill's neighbours (200 muscles, 6,910 pills, before the cull: 1,955 us
+// for two frames with one lane, 1,505 with two, 1,305 with four, 1,200 with eight;
+// strands and many scenes are fastest with one to four), and a contact CTA covers
+// fewer pills.
+constexpr int kSmallGroup = 16384, kEmitLanesSmall = 4, kContactPillsSmall = 64;
 constexpr int kMeshPerThread = 16;  // kLbsBatch vertices per round, 16 / kLbsBatch rounds
 
 size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -731,16 +828,17 @@ struct Fork {
 // Launch shape of one sequence: blocks per kernel kind over all its scenes.
 struct Shape {
     int tot[K_KINDS] = {};
-    int emit_mode = 1;  // pair search with the one-CTA grid: 1 unit / 2 chunk per warp
+    bool small = false;  // few pills (kSmallGroup)
     int threads = 0, smem = 16;
     bool cp = false, fused_grid = true;
+    int cluster = kGridClusterMax, cells_cap = 32, slice_cap = 32, groups_cap = 0;  // grid build: CTAs per scene, shared memory
 };
 
 // Device view of one scene for a frame of sub-step h (b.P.bq1 / bt1: the
 // scene's own target pose; the caller may point them elsewhere), and its
 // blocks per kernel kind.
 void fill_scene(BatchScene &b, int cnt[K_KINDS], viper_scene *s, const viper_batch_item &it, double h, bool cp,
-                int emit_ppw, bool small)
+                const Shape &sh)
 {
     memset(&b, 0, sizeof(b));
     b.P = s->P;
@@ -770,11 +868,12 @@ void fill_scene(BatchScene &b, int cnt[K_KINDS], viper_scene *s, const viper_bat
     const int nv = s->nv, ns = s->ns;
     cnt[K_ELEM] = cdiv(nv + ns, kElemThreads);
     cnt[K_PILL] = b.pills ? cdiv(ns, kElemThreads) : 0;
-    cnt[K_EMIT] = b.pills ? cdiv(ns, kEmitWarpsB * emit_ppw) : 0;  // about 0.4 emit_ppw work units per warp
+    cnt[K_EMIT] = b.pills ? cdiv((long long)ns * (sh.small ? kEmitLanesSmall : 1), 32 * kEmitWarpsB) : 0;
     cnt[K_SCAN] = b.pills ? 1 : 0;
+    cnt[K_GRID] = b.pills ? sh.cluster : 0;
     cnt[K_ROD] = s->n_items;
     cnt[K_CONTACT] = cp ? std::min(4 * device_sm_count(),
-                                   std::max(1, cdiv(ns + (s->n_planes > 0 ? nv : 0), small ? kContactPillsSmall : kElemThreads)))
+                                   std::max(1, cdiv(ns + (s->n_planes > 0 ? nv : 0), sh.small ? kContactPillsSmall : kElemThreads)))
                         : 0;
     cnt[K_END] = it.n_mesh > 0 ? std::max(1, cdiv(ns, kElemThreads)) : 1;
     cnt[K_MESH] = cdiv(it.n_mesh, kElemThreads * kMeshPerThread);
@@ -786,7 +885,12 @@ void shape_add(Shape &sh, const viper_scene *s, bool cp)
 {
     sh.cp = cp;
     sh.smem = std::max(sh.smem, cp ? s->smem_iter : s->smem_full);
-    if (s->ns > kGridMaxPills) sh.fused_grid = false;
+    if (cp && (s->flags & VIPER_FLAG_CONTACTS)) {
+        if (s->ns > kGridMaxPills) sh.fused_grid = false;
+        sh.cells_cap = std::max(sh.cells_cap, s->P.table / sh.cluster);
+        sh.slice_cap = std::max(sh.slice_cap, cdiv(s->ns, sh.cluster));
+        if (s->P.n_groups <= kGridGroupsMax) sh.groups_cap = std::max(sh.groups_cap, s->P.n_groups);
+    }
     sh.threads = s->block_threads;
 }
 
@@ -802,8 +906,10 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
                             : reinterpret_cast<const void *>(batch_rod_kernel<true>);
     if (raise_smem_limit(rod_fn, smem) != 0) return -1;
     if (cp && raise_smem_limit(reinterpret_cast<const void *>(batch_rod_first_kernel), smem) != 0) return -1;
-    const int grid_smem = kGridSmemBytes;
-    if (fused_grid && raise_smem_limit(reinterpret_cast<const void *>(batch_grid_kernel), grid_smem) != 0) return -1;
+    const int grid_smem = grid_smem_bytes(sh.cells_cap, sh.slice_cap, sh.groups_cap);
+    if (tot[K_GRID] > 0 && fused_grid &&
+        raise_smem_limit(reinterpret_cast<const void *>(batch_grid_kernel), grid_smem) != 0)
+        return -1;
     long long L = 0;
     auto go = [&](int cls, auto &&fn) {
         ProfScope ps(prof, cls);
@@ -813,7 +919,10 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
     auto broadphase = [&](cudaStream_t bs) {
         if (tot[K_PILL] <= 0) return;
         if (fused_grid) {
-            go(PROF_BROADPHASE, [&] { launch(batch_grid_kernel, tot[K_SCAN], kGridThreads, grid_smem, bs, A); });
+            go(PROF_BROADPHASE, [&] {
+                launch_clusters(batch_grid_kernel, tot[K_GRID], sh.cluster, kGridThreads, grid_smem, bs, A, sh.cells_cap,
+                                sh.slice_cap, sh.groups_cap);
+            });
         } else {
             go(PROF_BROADPHASE, [&] { launch(batch_bounds_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
             go(PROF_BROADPHASE, [&] { launch(batch_count_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
@@ -821,7 +930,7 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
             go(PROF_BROADPHASE, [&] { launch(batch_scatter_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
         }
         go(PROF_PAIRS, [&] {
-            launch(batch_emit_kernel, tot[K_EMIT], 32 * kEmitWarpsB, 0, bs, A, fused_grid ? sh.emit_mode : 0);
+            launch(sh.small ? batch_emit_kernel<kEmitLanesSmall> : batch_emit_kernel<1>, tot[K_EMIT], 32 * kEmitWarpsB, 0, bs, A);
         });
     };
     // the broadphase on a second branch beside the first sweep (not while profiling:
@@ -903,18 +1012,24 @@ int run_group(viper_batch *B, const viper_batch_item *items, const std::vector<i
     size_t bcur = 0;
     Shape sh;
     long long group_pills = 0;
+    int pill_scenes = 0, max_ns = 0, max_table = 0;
     for (int i : idx)
-        if (items[i].scene->flags & VIPER_FLAG_CONTACTS) group_pills += items[i].scene->ns;
-    const bool small_group = group_pills <= kEmitSmallGroup;
-    const int emit_ppw = small_group ? kEmitPillsPerWarpSmall : kEmitPillsPerWarp;
-    sh.emit_mode = small_group ? 1 : 2;
+        if (items[i].scene->flags & VIPER_FLAG_CONTACTS) {
+            const viper_scene *s = items[i].scene;
+            group_pills += s->ns;
+            ++pill_scenes;
+            max_ns = std::max(max_ns, s->ns);
+            max_table = std::max(max_table, s->P.table);
+        }
+    sh.cluster = grid_cluster(pill_scenes, max_ns, max_table);
+    sh.small = group_pills <= kSmallGroup;
     for (int c = 0; c < K_KINDS; ++c) off[c * (n + 1)] = 0;
     for (int k = 0; k < n; ++k) {
         const viper_batch_item &it = items[idx[k]];
         viper_scene *s = it.scene;
         BatchScene &b = hs[k];
         int cnt[K_KINDS];
-        fill_scene(b, cnt, s, it, h, cp, emit_ppw, small_group);
+        fill_scene(b, cnt, s, it, h, cp, sh);
         if (it.bone_quat && s->n_bones > 0) {  // this frame's target pose, from the call's table
             memcpy(hbq + bcur, it.bone_quat, sizeof(float4) * s->n_bones);
             memcpy(hbt + 3 * bcur, it.bone_trans, sizeof(float) * 3 * s->n_bones);
@@ -929,7 +1044,7 @@ int run_group(viper_batch *B, const viper_batch_item *items, const std::vector<i
     // a warp per contact pair shortens one scene's chain but multiplies the
     // lanes' work; once the scenes' contact passes fill the GPU, throughput
     // decides: one thread per pair
-    if (!small_group && sh.tot[K_CONTACT] > device_sm_count())
+    if (!sh.small && sh.tot[K_CONTACT] > device_sm_count())
         for (int k = 0; k < n; ++k) hs[k].P.contact_threads = 1;
 
     cudaStream_t st = B->stream;
@@ -969,12 +1084,11 @@ int self_batch_capture(viper_scene *s, float dt, int substeps, int iterations, c
     it.scene = s;
     const bool cp = scene_contact_path(s);
     int cnt[K_KINDS];
-    const bool small_group = s->ns <= kEmitSmallGroup;
-    const int emit_ppw = small_group ? kEmitPillsPerWarpSmall : kEmitPillsPerWarp;
-    fill_scene(*b, cnt, s, it, (double)dt / substeps, cp, emit_ppw, small_group);  // bones: the scene's own target pose
     Shape sh;
+    sh.small = s->ns <= kSmallGroup;
+    sh.cluster = grid_cluster(1, s->ns, s->P.table);
+    fill_scene(*b, cnt, s, it, (double)dt / substeps, cp, sh);  // bones: the scene's own target pose
     shape_add(sh, s, cp);
-    sh.emit_mode = small_group ? 1 : 2;
     for (int c = 0; c < K_KINDS; ++c) {
         off[2 * c] = 0;
         off[2 * c + 1] = cnt[c];

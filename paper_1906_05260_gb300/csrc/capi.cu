@@ -759,7 +759,6 @@ size_t viper_scene_footprint(const viper_scene_desc *d)
             b += 20 * cap + 16 * ns + 4 * (2 * ns) + 4 * (2 * table + 1) + 4 * 4096;  // pairs, their vertices, lambda
             b += 4 * (kBoundsWords + (size_t)broadphase_big_cap((int)ns));  // radius histogram, oversized pills
             b += (16 + 32) * nv;  // world and pill packs
-            b += 16 * (ns + ns / 32 + 1);  // pair-search chunk records
         }
     }
     return b;
@@ -837,6 +836,13 @@ int viper_scene_create(const viper_scene_desc *d, viper_scene **out)
     s->u_LC.resize(ns);
     s->u_group.resize(nr);
     for (int r = 0; r < nr; ++r) s->u_group[r] = d->group ? d->group[r] : r;
+    {  // numbered from 0: the device only compares them, and indexes tables by them
+        std::vector<int> ids(s->u_group);
+        std::sort(ids.begin(), ids.end());
+        ids.erase(std::unique(ids.begin(), ids.end()), ids.end());
+        for (int &g : s->u_group) g = (int)(std::lower_bound(ids.begin(), ids.end(), g) - ids.begin());
+        s->P.n_groups = (int)ids.size();
+    }
     s->u_origin.resize(nr);
     for (int r = 0; r < nr; ++r) {
         double c[3] = {0, 0, 0};
@@ -930,8 +936,6 @@ int viper_scene_create(const viper_scene_desc *d, viper_scene **out)
     A(P.big_list, pills ? P.big_cap : 1);
     A(P.cell_of, pills ? ns : 1); A(P.cell_pills, pills ? ns : 1);
     A(P.cell_sph, pills ? ns : 1); A(P.cell_grp, pills ? ns : 1);
-    // at most one chunk per occupied cell plus one per 32 pills
-    A(P.chunk_of, pills ? ns + ns / 32 + 1 : 1); A(P.n_chunks, 1);
     A(P.cell_count, P.table); A(P.cell_start, P.table + 1);
     A(s->d_scan_tmp, 4096);
     A(P.bar, 4); A(P.tile_sums, 1024);

@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(32 * kEmitWarps, 4) bp_emit_kernel(Params P)
     const unsigned int big = big_threshold(G.b_cut);
     const int nb = min(P.bp_hist[kRadBins], P.big_cap);
     for (int i = warp; i < nb; i += nwarps) emit_big(P, G, big, i, buf[wib], lane);
-    emit_pills(P, G, big, warp, nwarps, buf[wib], lane);
+    emit_pills<1>(P, G, big, P.ns, warp, nwarps, buf[wib], lane);
 }
 
 // ---------------------------------------------------------------- exclusive scan

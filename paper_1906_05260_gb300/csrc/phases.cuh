@@ -1129,28 +1129,33 @@ __device__ __forceinline__ bool spheres_overlap2(float4 na, float4 b)
     return __fadd_rn(__fadd_rn(ex, ey), ez) <= rs;
 }
 
-// Candidate pairs of the pills up to the cut, a thread per pill in cell order
-// (lane: entry p of the cell-order copies, pills p0 .. p0 + 31 per warp step).
+// Candidate pairs of the n pills in the cells, up to the cut, L lanes per pill in cell order
+// (a warp step takes entries p0 .. p0 + 32 / L - 1 of the cell-order copies).
 // Each tests the pills of its own cell after it and those of the 13 forward
 // neighbour cells (dz = 1; dz = 0, dy = 1; dz = dy = 0, dx = 1), so every pair
 // of pills in neighbouring cells is tested once.  Cells are numbered along x,
 // so these are five runs of the cell order: the rest of the own cell with the
-// next one, and four rows of three cells.  A lane walks its runs end to end,
-// four candidates a step; the warp takes the longest lane's number of steps.
-// Settled strands (300,000 pills, 8.8 million pairs): 216 us a search with the
-// oversized pills, against 469 us with fourteen lists each walked to the warp's
-// longest and the oversized pills tested against their whole list.
-__device__ __forceinline__ void emit_pills(const Params &P, const Grid &G, unsigned int big, int warp, int nwarps,
-                                           int *buf, int lane)
+// next one, and four rows of three cells.  A pill's lanes walk its runs end to
+// end, four candidates a lane and step; the warp takes the longest walk's
+// number of steps.
+// L = 1 where the pills fill the GPU: settled strands (300,000 pills, 8.8
+// million pairs) take 216 us a search with the oversized pills, against 469 us
+// with fourteen lists each walked to the warp's longest and the oversized pills
+// tested against their whole list.  More lanes shorten the walk where they do not.
+template <int L>
+__device__ __forceinline__ void emit_pills(const Params &P, const Grid &G, unsigned int big, int n, int warp,
+                                           int nwarps, int *buf, int lane)
 {
     const unsigned full = 0xffffffffu;
+    constexpr int kPer = 32 / L;  // pills per warp step
+    const int sub = lane % L;
     int *row = buf + lane * kLaneRow;
-    for (int p0 = warp * 32; p0 < P.ns; p0 += nwarps * 32) {
-        const int p = p0 + lane;
+    for (int p0 = warp * kPer; p0 < n; p0 += nwarps * kPer) {
+        const int p = p0 + lane / L;
         float4 na = make_float4(0.f, 0.f, 0.f, 0.f);
         int ga = 0, ia = 0, va = 0, cnt = 0;
         int q = 0, end = 0, q1 = 0, e1 = 0, q2 = 0, e2 = 0, q3 = 0, e3 = 0, q4 = 0, e4 = 0;
-        if (p < P.ns) {
+        if (p < n) {
             const float4 sa = P.cell_sph[p];
             if (!(__float_as_uint(sa.w) > big)) {
                 na = make_float4(-sa.x, -sa.y, -sa.z, sa.w);
@@ -1186,15 +1191,15 @@ __device__ __forceinline__ void emit_pills(const Params &P, const Grid &G, unsig
             int cg[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t)
-                if (q + t < end) {
-                    cs[t] = P.cell_sph[q + t];
-                    cg[t] = P.cell_grp[q + t];
+                if (q + t * L + sub < end) {
+                    cs[t] = P.cell_sph[q + t * L + sub];
+                    cg[t] = P.cell_grp[q + t * L + sub];
                 }
 #pragma unroll
             for (int t = 0; t < 4; ++t)
-                if (q + t < end && cg[t] != ga && spheres_overlap2(na, cs[t]) && !(__float_as_uint(cs[t].w) > big))
-                    row[cnt++] = q + t;
-            q += 4;
+                if (q + t * L + sub < end && cg[t] != ga && spheres_overlap2(na, cs[t]) && !(__float_as_uint(cs[t].w) > big))
+                    row[cnt++] = q + t * L + sub;
+            q += 4 * L;
             if (__any_sync(full, cnt > kLanePairs - 4)) {
                 flush_rows(P, buf, cnt, ia, va, lane);
                 cnt = 0;
@@ -1278,162 +1283,6 @@ __device__ __forceinline__ void emit_big(const Params &P, const Grid &G, unsigne
     }
     __syncwarp();
     if (cnt) flush_big(P, buf, cnt, gi, vi, lane);
-}
-
-// The chunk's pills (lane: entry pa of the cell order, sphere sa, group ga,
-// `own` when the lane holds a pill) against the neighbour list [d0, d1) by one
-// warp: the neighbour's pills are loaded 32 at a time from the cell-order
-// sphere / group copies (coalesced) into the warp's shared buffers (32 float4
-// + 32 int) and read back as broadcasts, STEP candidates per step.  SELF: the
-// list is the chunk's own cell from the chunk on, where only entries above pa
-// pair (each pair once); a forward neighbour's entries all lie above the
-// chunk's.  Steps without a hit in the warp cost one vote; hits are compacted
-// with a ballot and their output slots reserved with one atomic.
-template <int STEP, bool SELF, bool IDS>
-__device__ __forceinline__ void emit_block(const Params &P, int pa, bool own, float4 sa, int ga, int ia, int d0, int d1,
-                                           float4 *cbuf, int *gbuf, int *ibuf)
-{
-    const int lane = threadIdx.x & 31;
-    const unsigned full = 0xffffffffu;
-    for (int cb = d0; cb < d1; cb += 32) {
-        const int q = cb + lane;
-        __syncwarp();  // the previous block's reads are done
-        if (q < d1) {  // sphere and group of the block; with IDS the pill ids too (ready for the hits)
-            cbuf[lane] = P.cell_sph[q];
-            gbuf[lane] = P.cell_grp[q];
-            if (IDS) ibuf[lane] = P.cell_pills[q];
-        }
-        __syncwarp();
-        const int m = min(32, d1 - cb);
-        for (int j0 = 0; j0 < m; j0 += STEP) {
-            bool hit[STEP];
-            bool any = false;
-#pragma unroll
-            for (int t = 0; t < STEP; ++t) {
-                const int j = j0 + t;  // past m: no candidate (j & 31 is still a valid entry)
-                const float4 sj = cbuf[j & 31];
-                const int gj = gbuf[j & 31];
-                bool h = own && spheres_overlap(sa, sj) && gj != ga && j < m;
-                if (SELF) h = h && cb + j > pa;
-                hit[t] = h;
-                any = any || h;
-            }
-            if (!__any_sync(full, any)) continue;
-#pragma unroll
-            for (int t = 0; t < STEP; ++t) {
-                const unsigned hm = __ballot_sync(full, hit[t]);
-                if (hm) {
-                    int out = 0;
-                    if (lane == 0) out = atomicAdd(P.npairs, __popc(hm));
-                    out = __shfl_sync(full, out, 0);
-                    if (hit[t]) {
-                        const int idx = out + __popc(hm & ((1u << lane) - 1u));
-                        if (idx < P.max_pairs) {
-                            const int a = IDS ? ia : P.cell_pills[pa];
-                            const int b = IDS ? ibuf[j0 + t] : P.cell_pills[cb + j0 + t];
-                            P.pairs[idx] = make_int2(min(a, b), max(a, b));
-                            if (P.pair_v) P.pair_v[idx] = make_int2(P.seg_v0[min(a, b)], P.seg_v0[max(a, b)]);
-                            if (P.lam_pair) P.lam_pair[idx] = 0.f;
-                        }
-                    }
-                }
-            }
-        }
-    }
-}
-
-// Forward neighbour k < 13 of cell c (dz = 1: 9 cells; dz = 0, dy = 1: 3; dz = dy = 0, dx = 1),
-// or -1 outside the grid.
-__device__ __forceinline__ int forward_neighbour(const Grid &G, int c, int k)
-{
-    int dx, dy, dz;
-    if (k < 9) {
-        dx = k % 3 - 1; dy = k / 3 - 1; dz = 1;
-    } else if (k < 12) {
-        dx = k - 10; dy = 1; dz = 0;
-    } else {
-        dx = 1; dy = 0; dz = 0;
-    }
-    const int ix = c % G.dim[0], iy = (c / G.dim[0]) % G.dim[1], iz = c / (G.dim[0] * G.dim[1]);
-    const int x = ix + dx, y = iy + dy, z = iz + dz;
-    if (x < 0 || x >= G.dim[0] || y < 0 || y >= G.dim[1] || z >= G.dim[2]) return -1;
-    return x + G.dim[0] * (y + G.dim[1] * z);
-}
-
-// Candidate pairs of one chunk of up to 32 pills of a cell (chunk_of[q] =
-// (cell, chunk)) with one neighbour list, by one warp: work unit u = 14 q + k
-// pairs the chunk with the cell's forward neighbour k < 13, or with the rest of
-// its own cell from the chunk on (k = 13).  Every pair of pills of neighbouring
-// cells is visited once (as in emit_cell), and no unit is larger than one
-// chunk against one neighbour cell, so the units are balanced across warps.
-template <int STEP, class StartFn>
-__device__ __forceinline__ void emit_chunk(const Params &P, const Grid &G, int u, StartFn start, float4 *cbuf,
-                                           int *gbuf, int *ibuf)
-{
-    const int lane = threadIdx.x & 31;
-    const int k = u % kEmitUnits;
-    const int4 ch = P.chunk_of[u / kEmitUnits];
-    const int c = ch.x, o0 = ch.y, o1 = ch.z, cend = ch.w;
-    int d0, d1;
-    if (k == 13) {  // the own cell from this chunk on: pairs with pb > pa
-        d0 = o0;
-        d1 = cend;
-    } else {
-        const int d = forward_neighbour(G, c, k);
-        if (d < 0) return;
-        d0 = start(d);
-        d1 = start(d + 1);
-    }
-    if (d0 >= d1) return;  // uniform over the warp
-    const int pa = o0 + lane;
-    const bool own = pa < o1;
-    const float4 sa = own ? P.cell_sph[pa] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const int ga = own ? P.cell_grp[pa] : 0;
-    const int ia = own ? P.cell_pills[pa] : 0;  // latency bound: ids loaded beside the spheres
-    if (k == 13)
-        emit_block<STEP, true, true>(P, pa, own, sa, ga, ia, d0, d1, cbuf, gbuf, ibuf);
-    else
-        emit_block<STEP, false, true>(P, pa, own, sa, ga, ia, d0, d1, cbuf, gbuf, ibuf);
-}
-
-// All 14 neighbour lists of chunk q by one warp (the same pairs as the 14 units
-// of emit_chunk): lanes 0..13 look up the lists' ranges at once, then the warp
-// walks the non-empty ones.  Fewer, longer units: for many scenes at once, where
-// each unit's chain of dependent loads, not its tests, sets the time.
-template <int STEP, class StartFn>
-__device__ __forceinline__ void emit_chunk_all(const Params &P, const Grid &G, int q, StartFn start, float4 *cbuf,
-                                               int *gbuf, int *ibuf)
-{
-    const int lane = threadIdx.x & 31;
-    const unsigned full = 0xffffffffu;
-    const int4 ch = P.chunk_of[q];
-    const int c = ch.x, o0 = ch.y, o1 = ch.z, cend = ch.w;
-    int d0 = 0, d1 = 0;
-    if (lane == 13) {  // the own cell from this chunk on
-        d0 = o0;
-        d1 = cend;
-    } else if (lane < 13) {
-        const int d = forward_neighbour(G, c, lane);
-        if (d >= 0) {
-            d0 = start(d);
-            d1 = start(d + 1);
-        }
-    }
-    const int pa = o0 + lane;
-    const bool own = pa < o1;
-    const float4 sa = own ? P.cell_sph[pa] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const int ga = own ? P.cell_grp[pa] : 0;
-    unsigned lists = __ballot_sync(full, lane < 14 && d1 > d0);
-    while (lists) {
-        const int k = __ffs(lists) - 1;
-        lists &= lists - 1;
-        const int b0 = __shfl_sync(full, d0, k), b1 = __shfl_sync(full, d1, k);
-        // throughput bound (many scenes): pill ids loaded only for the hits
-        if (k == 13)
-            emit_block<STEP, true, false>(P, pa, own, sa, ga, 0, b0, b1, cbuf, gbuf, ibuf);
-        else
-            emit_block<STEP, false, false>(P, pa, own, sa, ga, 0, b0, b1, cbuf, gbuf, ibuf);
-    }
 }
 
 // ================================================================ contacts

@@ -68,6 +68,7 @@ struct Params {
     // fraction t, 0); b0 < 0: not warm-started; null: no warm start
     const float4 *warm;
     const int *seg_v0, *vtx_seg, *seg_group;
+    int n_groups;  // a scene's groups are numbered 0 .. n_groups - 1
     // Vertex positions are stored relative to a per-rod FP32 origin (the rod's
     // rest centroid) so that differences along a rod keep full precision far
     // from the world origin; world = local + rod_origin[rod_of_v[v]].
@@ -121,8 +122,6 @@ struct Params {
     int *cell_of, *cell_count, *cell_start, *cell_pills;
     float4 *cell_sph;  // bounding spheres in cell order
     int *cell_grp;     // collision groups in cell order
-    int4 *chunk_of;    // pair-search chunks of 32 pills: (cell, first, end, cell end) in cell order, from the one-CTA grid build
-    int *n_chunks;
     int table;
     Grid *grid;
     int *err;
