@@ -1,5 +1,6 @@
 // capi.cu -- C ABI of the VIPER library: scene creation (rest precompute,
 // rod packing), frame stepping with CUDA-graph replay, skinning and state I/O.
+#include <cuda.h>
 #include <math.h>
 #include <string.h>
 
@@ -85,6 +86,38 @@ bool is_device_ptr(const void *p)
         return false;
     }
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// Whether a kernel on the current device can use p as an array of `bytes` bytes of
+// 16-byte elements: device memory of this device, aligned, and all of it inside
+// one allocation (as far as the driver knows allocations).  Anything else
+// (host, managed or another device's memory, odd addresses) goes through copies.
+bool device_array(const void *p, size_t bytes)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    int dev = -1;
+    if (a.type != cudaMemoryTypeDevice || (reinterpret_cast<uintptr_t>(p) & 15u) != 0 ||
+        cudaGetDevice(&dev) != cudaSuccess || a.device != dev)
+        return false;
+    using AddressRange = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const AddressRange range = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult qr;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &qr) != cudaSuccess ||
+            qr != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<AddressRange>(fn);
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = (CUdeviceptr) reinterpret_cast<uintptr_t>(p);
+    return range && range(&base, &size, at) == CUDA_SUCCESS && at + bytes <= base + size;
 }
 
 // Device address of page-locked host memory (cudaHostAlloc / cudaHostRegister),
@@ -800,8 +833,8 @@ int viper_scene_create(const viper_scene_desc *d, viper_scene **out)
     if (cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming) != cudaSuccess) return fail(VIPER_ECUDA);
     if (cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess) return fail(VIPER_ECUDA);
     // mapped, so that the multi-scene step can write it from the device
-    if (cudaHostAlloc((void **)&s->h_err, sizeof(int), cudaHostAllocMapped) != cudaSuccess) return fail(VIPER_ECUDA);
-    *s->h_err = 0;
+    if (cudaHostAlloc((void **)&s->h_err, 2 * sizeof(int), cudaHostAllocMapped) != cudaSuccess) return fail(VIPER_ECUDA);
+    s->h_err[0] = s->h_err[1] = 0;
     if (cudaHostGetDevicePointer((void **)&s->d_herr, s->h_err, 0) != cudaSuccess) return fail(VIPER_ECUDA);
 
     // ---- rest data in FP64, caller order (Sec. 4 discretisation), kept for activation
@@ -1300,35 +1333,73 @@ int viper_skin(viper_scene *s, int n, const float *rest4, const int *idx4, const
     return cudaGetLastError() == cudaSuccess ? VIPER_OK : VIPER_ECUDA;
 }
 
+// Waits for the stream, on which the error word has been taken (take_error), and
+// reports it: overflow once; non-finite stays latched until a new state is set.
+static int taken_error(viper_scene *s)
+{
+    VCHECK(cudaStreamSynchronize(s->stream));
+    s->latched |= s->h_err[1] | s->h_err[0];
+    const int code = decode_err(s->latched);
+    s->latched &= ERR_NONFINITE;
+    if (!(s->latched & ERR_NONFINITE)) s->h_err[0] = 0;
+    return code;
+}
+
 int viper_get_state(viper_scene *s, float *x4, float *v4, float *q4, float *w4)
 {
     if (!s) return VIPER_EINVAL;
     float *dst[4] = {x4, v4, q4, w4};
+    StateArrays direct = {};
+    bool any = false;
     for (int w = 0; w < 4; ++w) {
         if (!dst[w]) continue;
-        int n = w < 2 ? s->nv : s->ns;
+        const size_t bytes = sizeof(float4) * (size_t)(w < 2 ? s->nv : s->ns);
+        // written directly unless it overlaps another of the arrays (the later one
+        // then holds, as copies one after the other leave it)
+        bool alone = device_array(dst[w], bytes);
+        for (int u = 0; u < 4 && alone; ++u) {
+            const size_t ub = sizeof(float4) * (size_t)(u < 2 ? s->nv : s->ns);
+            const uintptr_t a = reinterpret_cast<uintptr_t>(dst[w]), b = reinterpret_cast<uintptr_t>(dst[u]);
+            if (u != w && dst[u] && a < b + ub && b < a + bytes) alone = false;
+        }
+        if (alone) {
+            direct.p[w] = reinterpret_cast<float4 *>(dst[w]);
+            any = true;
+            continue;
+        }
         launch_state_out(s, w, s->stage4);
-        VCHECK(cudaMemcpyAsync(dst[w], s->stage4, sizeof(float4) * n, cudaMemcpyDefault, s->stream));
+        VCHECK(cudaMemcpyAsync(dst[w], s->stage4, bytes, cudaMemcpyDefault, s->stream));
     }
-    VCHECK(cudaStreamSynchronize(s->stream));
-    return viper_sync(s);
+    if (any)
+        launch_state_out_all(s, direct);
+    else
+        launch_take_error(s);
+    VCHECK(cudaGetLastError());
+    return taken_error(s);
 }
 
 int viper_set_state(viper_scene *s, const float *x4, const float *v4, const float *q4, const float *w4)
 {
     if (!s) return VIPER_EINVAL;
     const float *src[4] = {x4, v4, q4, w4};
+    StateArrays direct = {};
+    bool any = false;
     for (int w = 0; w < 4; ++w) {
         if (!src[w]) continue;
-        int n = w < 2 ? s->nv : s->ns;
-        VCHECK(cudaMemcpyAsync(s->stage4, src[w], sizeof(float4) * n, cudaMemcpyDefault, s->stream));
+        const size_t bytes = sizeof(float4) * (size_t)(w < 2 ? s->nv : s->ns);
+        if (device_array(src[w], bytes)) {
+            direct.p[w] = const_cast<float4 *>(reinterpret_cast<const float4 *>(src[w]));
+            any = true;
+            continue;
+        }
+        VCHECK(cudaMemcpyAsync(s->stage4, src[w], bytes, cudaMemcpyDefault, s->stream));
         launch_state_in(s, w, s->stage4);
     }
-    VCHECK(cudaStreamSynchronize(s->stream));
+    if (any) launch_state_in_all(s, direct);
     // a new state lifts the non-finite quarantine
     VCHECK(cudaMemsetAsync(s->P.err, 0, sizeof(int), s->stream));
     VCHECK(cudaStreamSynchronize(s->stream));
-    *s->h_err = 0;
+    s->h_err[0] = 0;
     s->latched = 0;
     return VIPER_OK;
 }
@@ -1336,18 +1407,9 @@ int viper_set_state(viper_scene *s, const float *x4, const float *v4, const floa
 int viper_sync(viper_scene *s)
 {
     if (!s) return VIPER_EINVAL;
-    VCHECK(cudaStreamSynchronize(s->stream));
-    int e = 0;
-    VCHECK(cudaMemcpy(&e, s->P.err, sizeof(int), cudaMemcpyDeviceToHost));
-    s->latched |= e | *s->h_err;
-    int code = decode_err(s->latched);
-    // overflow is reported once; non-finite stays latched until a new state is set
-    s->latched &= ERR_NONFINITE;
-    if (!(s->latched & ERR_NONFINITE)) {
-        VCHECK(cudaMemset(s->P.err, 0, sizeof(int)));
-        *s->h_err = 0;
-    }
-    return code;
+    launch_take_error(s);
+    VCHECK(cudaGetLastError());
+    return taken_error(s);
 }
 
 int viper_get_pairs(viper_scene *s, int *pairs, int cap, int *n_pairs)

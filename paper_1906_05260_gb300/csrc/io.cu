@@ -83,38 +83,28 @@ void launch_lbs(viper_scene *s, int n, const float4 *rest, const int4 *idx, cons
 // ------------------------------------------------------------------ state I/O
 // which: 0 = X (x, y, z, radius), 1 = V (v, d radius/dt), 2 = Q, 3 = W.
 // Internally vertices carry the scale s; the caller sees radius = s * rbar.
-__global__ void state_out_kernel(Params P, int which, const int *__restrict__ perm, float4 *__restrict__ dst)
+__device__ __forceinline__ float4 state_out(const Params &P, int which, int i)
 {
-    int n = which < 2 ? P.nv : P.ns;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (which == 2) return P.Q[i];
+    if (which == 3) return P.W[i];
     float4 v;
     if (which == 0) {
         v = P.X[i];
-        float4 o = P.rod_origin[P.rod_of_v[i]];
+        const float4 o = P.rod_origin[P.rod_of_v[i]];
         v.x = __fadd_rn(v.x, o.x);
         v.y = __fadd_rn(v.y, o.y);
         v.z = __fadd_rn(v.z, o.z);
-        v.w *= P.RV0[i].w;
-    } else if (which == 1) {
-        v = P.V[i];
-        v.w *= P.RV0[i].w;
-    } else if (which == 2) {
-        v = P.Q[i];
     } else {
-        v = P.W[i];
+        v = P.V[i];
     }
-    dst[perm[i]] = v;
+    v.w *= P.RV0[i].w;
+    return v;
 }
 
-__global__ void state_in_kernel(Params P, int which, const int *__restrict__ perm, const float4 *__restrict__ src)
+__device__ __forceinline__ void state_in(const Params &P, int which, int i, float4 v)
 {
-    int n = which < 2 ? P.nv : P.ns;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float4 v = src[perm[i]];
     if (which == 0) {
-        float4 o = P.rod_origin[P.rod_of_v[i]];
+        const float4 o = P.rod_origin[P.rod_of_v[i]];
         v.x = __fsub_rn(v.x, o.x);
         v.y = __fsub_rn(v.y, o.y);
         v.z = __fsub_rn(v.z, o.z);
@@ -128,6 +118,64 @@ __global__ void state_in_kernel(Params P, int which, const int *__restrict__ per
     } else {
         v.w = 0.f;
         P.W[i] = v;
+    }
+}
+
+__global__ void state_out_kernel(Params P, int which, const int *__restrict__ perm, float4 *__restrict__ dst)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < (which < 2 ? P.nv : P.ns)) dst[perm[i]] = state_out(P, which, i);
+}
+
+__global__ void state_in_kernel(Params P, int which, const int *__restrict__ perm, const float4 *__restrict__ src)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < (which < 2 ? P.nv : P.ns)) state_in(P, which, i, src[perm[i]]);
+}
+
+// The error word for the host: copied to `mirror` and cleared, except for a
+// non-finite state, which stays until a new state is set.
+__device__ __forceinline__ void take_error(int *err, int *mirror)
+{
+    const int e = *(volatile int *)err;
+    *(volatile int *)mirror = e;
+    if (!(e & ERR_NONFINITE)) *err = 0;
+}
+
+__global__ void take_error_kernel(int *err, int *mirror) { take_error(err, mirror); }
+
+// All of the state in one launch, straight between the caller's device arrays
+// (null: left out) and the scene's: a thread per vertex, then per segment.  The
+// transfer is bound by its launches, not its bytes: eight copies and kernels,
+// and the error word's own copy and reset, took 73 us more of a
+// 512-vertex scene's set, two frames and get (341 us) than this.
+__global__ void state_out_all_kernel(Params P, const int *__restrict__ vperm, const int *__restrict__ sperm, StateArrays a,
+                                     int *mirror)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) take_error(P.err, mirror);
+    if (i < P.nv) {
+        const int k = vperm[i];
+        if (a.p[0]) a.p[0][k] = state_out(P, 0, i);
+        if (a.p[1]) a.p[1][k] = state_out(P, 1, i);
+    } else if (i < P.nv + P.ns) {
+        const int j = i - P.nv, k = sperm[j];
+        if (a.p[2]) a.p[2][k] = state_out(P, 2, j);
+        if (a.p[3]) a.p[3][k] = state_out(P, 3, j);
+    }
+}
+
+__global__ void state_in_all_kernel(Params P, const int *__restrict__ vperm, const int *__restrict__ sperm, StateArrays a)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < P.nv) {
+        const int k = vperm[i];
+        if (a.p[0]) state_in(P, 0, i, a.p[0][k]);
+        if (a.p[1]) state_in(P, 1, i, a.p[1][k]);
+    } else if (i < P.nv + P.ns) {
+        const int j = i - P.nv, k = sperm[j];
+        if (a.p[2]) state_in(P, 2, j, a.p[2][k]);
+        if (a.p[3]) state_in(P, 3, j, a.p[3][k]);
     }
 }
 
@@ -151,6 +199,24 @@ void launch_state_in(viper_scene *s, int which, const float4 *src)
 {
     int n = which < 2 ? s->nv : s->ns;
     state_in_kernel<<<(n + 255) / 256, 256, 0, s->ls>>>(s->P, which, which < 2 ? s->d_vperm : s->d_sperm, src);
+    s->launches++;
+}
+
+void launch_state_out_all(viper_scene *s, const StateArrays &a)
+{
+    state_out_all_kernel<<<(s->nv + s->ns + 255) / 256, 256, 0, s->ls>>>(s->P, s->d_vperm, s->d_sperm, a, s->d_herr + 1);
+    s->launches++;
+}
+
+void launch_state_in_all(viper_scene *s, const StateArrays &a)
+{
+    state_in_all_kernel<<<(s->nv + s->ns + 255) / 256, 256, 0, s->ls>>>(s->P, s->d_vperm, s->d_sperm, a);
+    s->launches++;
+}
+
+void launch_take_error(viper_scene *s)
+{
+    take_error_kernel<<<1, 1, 0, s->ls>>>(s->P.err, s->d_herr + 1);
     s->launches++;
 }
 

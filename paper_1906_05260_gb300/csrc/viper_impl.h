@@ -211,7 +211,8 @@ struct viper_scene {
     cudaEvent_t ev_act = nullptr;
     bool act_on = false;
     std::vector<int> u_xs_vert, u_xs_seg;  // bundle cross-section members, caller numbering
-    // pinned, mapped host mirror of the device error word (read without a stream sync)
+    // pinned, mapped host mirrors of the device error word: [0] written at the end of
+    // every frame (read without a stream sync), [1] when it is taken (take_error)
     int *h_err = nullptr;
     int *d_herr = nullptr;  // its device address
     void *self_table = nullptr;  // one-scene table of the multi-scene kernels (graph path)
@@ -275,6 +276,13 @@ void launch_warm(viper_scene *s);
 void launch_activation(viper_scene *s);
 void launch_state_out(viper_scene *s, int which, float4 *dst);
 void launch_state_in(viper_scene *s, int which, const float4 *src);
+// The caller's device arrays of a state (x4, v4, q4, w4; null: left out).
+struct StateArrays {
+    float4 *p[4];
+};
+void launch_state_out_all(viper_scene *s, const StateArrays &a);  // and the error word to h_err[1] (take_error)
+void launch_state_in_all(viper_scene *s, const StateArrays &a);
+void launch_take_error(viper_scene *s);
 void launch_predicted_out(viper_scene *s, float4 *dst, float *rbar);
 int configure_rod_kernels(int smem_bytes);
 // scene helpers shared with the multi-scene step (capi.cu)
