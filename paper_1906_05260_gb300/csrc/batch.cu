@@ -13,7 +13,7 @@
 //   grid (one CTA per scene: bounds, counts, scan, scatter) | pair search |
 //   contact | {sweep | contact} x (I - 1)
 // and one velocity update after the last substep: S (2 I + 2) + 1 launches.
-// Without contacts: one full shared-memory rod launch per substep.  After the
+// Without contacts: one launch for all substeps.  After the
 // substeps one launch builds the skinning frames, hands the bone pose on and
 // mirrors the error word to the host; one more skins every mesh.
 //
@@ -573,18 +573,26 @@ __device__ __forceinline__ bool packs_used(const Params &P, bool first_sweep)
     return !first_sweep && P.XW && *P.npairs >= kPackPairs * P.ns;
 }
 
-// One colour sweep of every work item (contact path): FULL = false, or the
-// whole substep with all iterations (no contacts): FULL = true.
-template <bool FULL>
-__global__ void __launch_bounds__(256, 2) batch_rod_kernel(BatchArgs A, int n_iter, int first, int apply, float tau)
+// One colour sweep of every work item (contact path).
+__global__ void __launch_bounds__(256, 2) batch_rod_kernel(BatchArgs A, int first, int apply)
 {
     __shared__ BatchScene sb;
     extern __shared__ float4 smem[];
     int local, nblk;
     batch_enter(A, K_ROD, sb, local, nblk);
     // read after rod_item's first barrier
-    if (!FULL && threadIdx.x == 0 && !packs_used(sb.P, first != 0)) sb.P.XW = nullptr;
-    rod_item<FULL>(sb.P, local, n_iter, first != 0, apply != 0, tau, smem);
+    if (threadIdx.x == 0 && !packs_used(sb.P, first != 0)) sb.P.XW = nullptr;
+    rod_item(sb.P, local, first != 0, apply != 0, smem);
+}
+
+// Every substep of the frame (no contacts).
+__global__ void __launch_bounds__(256, 2) batch_rod_frame_kernel(BatchArgs A, int substeps, int n_iter)
+{
+    __shared__ BatchScene sb;
+    extern __shared__ float4 smem[];
+    int local, nblk;
+    batch_enter(A, K_ROD, sb, local, nblk);
+    rod_frame_item(sb.P, local, substeps, n_iter, smem);
 }
 
 // Jacobi contact pass (Sec. 7.2) after the sweep `first`: pairs, then half-plane
@@ -902,8 +910,8 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
     const int *tot = sh.tot;
     const int threads = sh.threads, smem = sh.smem;
     const bool cp = sh.cp, fused_grid = sh.fused_grid;
-    const void *rod_fn = cp ? reinterpret_cast<const void *>(batch_rod_kernel<false>)
-                            : reinterpret_cast<const void *>(batch_rod_kernel<true>);
+    const void *rod_fn = cp ? reinterpret_cast<const void *>(batch_rod_kernel)
+                            : reinterpret_cast<const void *>(batch_rod_frame_kernel);
     if (raise_smem_limit(rod_fn, smem) != 0) return -1;
     if (cp && raise_smem_limit(reinterpret_cast<const void *>(batch_rod_first_kernel), smem) != 0) return -1;
     const int grid_smem = grid_smem_bytes(sh.cells_cap, sh.slice_cap, sh.groups_cap);
@@ -952,7 +960,7 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
                     return -1;
                 broadphase(fork->side);
                 if (cudaEventRecord(fork->ev_join, fork->side) != cudaSuccess) return -1;
-                go(PROF_ROD, [&] { launch(batch_rod_kernel<false>, tot[K_ROD], threads, smem, st, A, 1, 1, 0, tau); });
+                go(PROF_ROD, [&] { launch(batch_rod_kernel, tot[K_ROD], threads, smem, st, A, 1, 0); });
                 if (cudaStreamWaitEvent(st, fork->ev_join, 0) != cudaSuccess) return -1;
             } else {
                 go(PROF_ROD, [&] { launch(batch_rod_first_kernel, tot[K_ROD], threads, smem, st, A, k > 0 ? 1 : 0, tau); });
@@ -960,21 +968,19 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
             }
             contact(1);
             for (int i = 1; i < iterations; ++i) {
-                go(PROF_ROD, [&] { launch(batch_rod_kernel<false>, tot[K_ROD], threads, smem, st, A, 1, 0, 1, tau); });
+                go(PROF_ROD, [&] { launch(batch_rod_kernel, tot[K_ROD], threads, smem, st, A, 0, 1); });
                 contact(0);
             }
             if (tot[K_BUNDLE] > 0)
                 go(PROF_ELEM, [&] { launch(batch_bundle_kernel, tot[K_BUNDLE], kElemThreads, 0, st, A); });
         }
         go(PROF_ELEM, [&] { launch(batch_finish_kernel, tot[K_ELEM], kElemThreads, 0, st, A, 1); });
+    } else if (!cp) {
+        go(PROF_ROD, [&] { launch(batch_rod_frame_kernel, tot[K_ROD], threads, smem, st, A, substeps, iterations); });
     } else {
+        // contact path without iterations: prediction, broadphase, velocity update
         for (int k = 0; k < substeps; ++k) {
             const float tau = (float)((double)(k + 1) / substeps);  // as the one-scene path
-            if (!cp) {
-                go(PROF_ROD, [&] { launch(batch_rod_kernel<true>, tot[K_ROD], threads, smem, st, A, iterations, 1, 0, tau); });
-                continue;
-            }
-            // contact path without iterations: prediction, broadphase, velocity update
             go(PROF_ELEM, [&] { launch(batch_predict_kernel, tot[K_ELEM], kElemThreads, 0, st, A, tau); });
             broadphase(st);
             go(PROF_ELEM, [&] { launch(batch_finish_kernel, tot[K_ELEM], kElemThreads, 0, st, A, 0); });

@@ -556,6 +556,8 @@ void enqueue_frame(viper_scene *s, float dt, int substeps, int iterations)
     const int nv = s->nv, ns = s->ns;
     if (P.warm && s->mode != VIPER_SOLVER_FRAME) launch_warm(s);  // the frame kernel warm-starts itself
     if (s->mode == VIPER_SOLVER_FRAME) substeps_frame(s, substeps, iterations);
+    // without contacts nothing couples the shared-memory rods to the others: all their substeps at once
+    if (s->mode == VIPER_SOLVER_BATCHED && !cp) launch_rod_frame(s, substeps, iterations);
     for (int k = 0; k < substeps && s->mode != VIPER_SOLVER_FRAME; ++k) {
         P.tau = (float)((double)(k + 1) / substeps);
         if (s->mode == VIPER_SOLVER_PLAIN) {
@@ -571,7 +573,6 @@ void enqueue_frame(viper_scene *s, float dt, int substeps, int iterations)
             if (iterations > 0) launch_bundles(s);
             launch_finish(s, 0, nv, 0, ns, false);
         } else if (!cp) {
-            launch_rod_full(s, iterations);
             if (s->resident_nv < nv) {
                 launch_predict(s, s->resident_nv, nv, s->resident_ns, ns, false);
                 for (int it = 0; it < iterations; ++it)

@@ -6,12 +6,13 @@
 //  * seg_colour_kernel / vtx_colour_kernel: one launch per constraint colour
 //    (even segments, odd segments, even interior vertices, odd interior
 //    vertices), one thread per constraint, state in HBM -- the plain path.
-//  * rod_kernel<FULL>: a CTA owns a packed work item of whole rods, stages
-//    their float4 state in shared memory with coalesced 128-bit loads, runs
-//    every colour sweep of the substep (FULL: prediction, all iterations and
-//    the velocity update; otherwise one iteration between contact passes) with
-//    each thread keeping its constraints' rest data and XPBD multipliers in
-//    registers, and writes the state back with 128-bit stores.
+//  * rod_kernel: a CTA owns a packed work item of whole rods, stages their float4
+//    state in shared memory with coalesced 128-bit loads, runs one iteration
+//    between contact passes with each thread keeping its constraints' rest data
+//    and XPBD multipliers in registers, and writes the state back with 128-bit
+//    stores.
+//  * rod_frame_kernel: the same for every substep of a frame without contacts
+//    (prediction, all iterations and the velocity update), state staged once.
 #include "phases.cuh"
 
 namespace viper {
@@ -178,11 +179,16 @@ __global__ void bundle_kernel(Params P)
 }
 
 // ------------------------------------------------------------------ shared-memory rods
-template <bool FULL>
-__global__ void __launch_bounds__(256) rod_kernel(Params P, int n_iter, int first, int apply)
+__global__ void __launch_bounds__(256) rod_kernel(Params P, int first, int apply)
 {
     extern __shared__ float4 smem[];
-    rod_item<FULL>(P, blockIdx.x, n_iter, first != 0, apply != 0, P.tau, smem);
+    rod_item(P, blockIdx.x, first != 0, apply != 0, smem);
+}
+
+__global__ void __launch_bounds__(256) rod_frame_kernel(Params P, int substeps, int n_iter)
+{
+    extern __shared__ float4 smem[];
+    rod_frame_item(P, blockIdx.x, substeps, n_iter, smem);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -254,11 +260,11 @@ void launch_bundles(viper_scene *s)
     s->launches++;
 }
 
-void launch_rod_full(viper_scene *s, int n_iter)
+void launch_rod_frame(viper_scene *s, int substeps, int n_iter)
 {
     if (s->n_items <= 0) return;
     ProfScope ps(s, PROF_ROD);
-    rod_kernel<true><<<s->n_items, s->block_threads, s->smem_full, s->ls>>>(s->P, n_iter, 1, 0);
+    rod_frame_kernel<<<s->n_items, s->block_threads, s->smem_full, s->ls>>>(s->P, substeps, n_iter);
     s->launches++;
 }
 
@@ -276,15 +282,15 @@ void launch_rod_iter(viper_scene *s, bool first, bool apply)
 {
     if (s->n_items <= 0) return;
     ProfScope ps(s, PROF_ROD);
-    rod_kernel<false><<<s->n_items, s->block_threads, s->smem_iter, s->ls>>>(contact_path_params(s), 1,
-                                                                                 first ? 1 : 0, apply ? 1 : 0);
+    rod_kernel<<<s->n_items, s->block_threads, s->smem_iter, s->ls>>>(contact_path_params(s), first ? 1 : 0,
+                                                                      apply ? 1 : 0);
     s->launches++;
 }
 
 int configure_rod_kernels(int smem_full)
 {
-    int e1 = raise_smem_limit(reinterpret_cast<const void *>(rod_kernel<true>), smem_full);
-    int e2 = raise_smem_limit(reinterpret_cast<const void *>(rod_kernel<false>), smem_full);
+    int e1 = raise_smem_limit(reinterpret_cast<const void *>(rod_frame_kernel), smem_full);
+    int e2 = raise_smem_limit(reinterpret_cast<const void *>(rod_kernel), smem_full);
     return (e1 == 0 && e2 == 0) ? 0 : -1;
 }
 

@@ -258,7 +258,7 @@ struct ProfScope {
 void launch_predict(viper_scene *s, int v_begin, int v_end, int s_begin, int s_end, bool contact_path);
 void launch_finish(viper_scene *s, int v_begin, int v_end, int s_begin, int s_end, bool apply);
 void launch_colour(viper_scene *s, int colour, const int *list, int n);
-void launch_rod_full(viper_scene *s, int n_iter);
+void launch_rod_frame(viper_scene *s, int substeps, int n_iter);
 void launch_rod_iter(viper_scene *s, bool first, bool apply);
 void launch_apply(viper_scene *s, int v_begin, int v_end);
 void launch_broadphase(viper_scene *s);
