@@ -184,8 +184,8 @@ __global__ void __launch_bounds__(kElemThreads) batch_scatter_kernel(BatchArgs A
     }
 }
 
-// Candidate pairs, L lanes per pill (see emit_pills; no oversized pills here:
-// the cell is sized for the largest).
+// Candidate pairs: a warp per oversized pill (with the cluster's grid), then L
+// lanes per pill (see emit_big, emit_pills).
 template <int L>
 __global__ void __launch_bounds__(32 * kEmitWarpsB) batch_emit_kernel(BatchArgs A)
 {
@@ -197,8 +197,12 @@ __global__ void __launch_bounds__(32 * kEmitWarpsB) batch_emit_kernel(BatchArgs 
     const Grid G = *P.grid;
     if (G.pad) return;  // no valid grid: no candidates (uniform over the CTA)
     const int wib = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = local * kEmitWarpsB + wib, nwarps = nblk * kEmitWarpsB;
     const int n = P.cell_start[grid_cells(&G, P.table)];  // pills in the cells
-    emit_pills<L>(P, G, 0xffffffffu, n, local * kEmitWarpsB + wib, nblk * kEmitWarpsB, buf[wib], threadIdx.x & 31);
+    const unsigned int big = big_threshold(G.b_cut);
+    const int nb = G.b_cut < kRadBins - 1 ? min(P.bp_hist[kRadBins], P.big_cap) : 0;
+    for (int i = warp; i < nb; i += nwarps) emit_big(P, G, big, i, buf[wib], lane);
+    emit_pills<L>(P, G, big, n, warp, nwarps, buf[wib], lane);
 }
 
 // ---------------------------------------------------------------- one scene's grid by one cluster
@@ -261,8 +265,11 @@ __device__ __forceinline__ int cluster_add(unsigned addr, int v)
 // the largest pill, nine times the smallest) held 180 candidates a pill, nearly
 // all of the pill's own muscle.
 //
+// Where at most kGridFew stay, they are put in one cell, and the pair search tests
+// them all; the steps below are left out.
+//
 // The build is a chain of dependent phases, too short for a launch each and too
-// long for one CTA (10,080 pills: 38.5 us by one CTA of 512 threads, 18.4 by eight).
+// long for one CTA (10,080 pills: 38.5 us by one CTA of 512 threads, 12 by eight).
 // The cluster splits the pills into slices and the cells into ranges of 2^sh,
 // one of each per CTA, all in shared memory: spheres and the pills' cells in
 // their slice, counts and starts in the range's owner.  Counting a pill returns
@@ -270,14 +277,16 @@ __device__ __forceinline__ int cluster_add(unsigned addr, int v)
 // The CTAs meet five times (boxes, bounds, counts, range totals, end).
 // Dynamic shared memory: slice_cap spheres, cells (first the pills' vertices) and
 // places (first their groups), cells_cap cell counts (the table's share of a CTA, a
-// power of two), and per group this CTA's and the scene's box (6 words each).
-constexpr int kGridThreads = 512, kGridClusterMax = 8, kGridCellsMax = 16384, kGridSliceMax = 6144;
-constexpr int kGridMaxPills = kGridClusterMax * kGridSliceMax;  // 49,152: table of 131,072 cells = 8 x kGridCellsMax
-constexpr int kGridGroupsMax = 512;
+// power of two), and per group this CTA's and the scene's box.
+constexpr int kGridThreads = 512, kGridClusterMax = 8, kGridCellsMax = 16384, kGridSliceMax = 5120;
+constexpr int kGridMaxPills = kGridClusterMax * kGridSliceMax;  // 40,960: table of 131,072 cells = 8 x kGridCellsMax
+constexpr int kGridGroupsMax = 512, kGridFew = 128;
 inline int grid_smem_bytes(int cells_cap, int slice_cap, int groups_cap)
 {
-    return (16 + 4 + 4) * slice_cap + 4 * cells_cap + 48 * groups_cap;
+    return (16 + 4 + 4) * slice_cap + 4 * cells_cap + 64 * groups_cap;
 }
+static_assert((16 + 4 + 4) * kGridSliceMax + 4 * kGridCellsMax + 64 * kGridGroupsMax + 6144 <= 227 * 1024,
+              "the largest scene's grid fits a CTA's shared memory (6 KB of it static)");
 
 // Half-width of the box of sphere sp in the cull: its radius and a margin far above
 // the rounding of the box and of spheres_overlap.
@@ -286,69 +295,90 @@ __device__ __forceinline__ float cull_reach(float4 sp)
     return 1.0078125f * fabsf(sp.w) + 1e-6f * (fabsf(sp.x) + fabsf(sp.y) + fabsf(sp.z));
 }
 
+// Whether all bounds are finite, as make_grid_from requires them.
+__device__ __forceinline__ bool finite_bounds(const unsigned *bounds)
+{
+    bool ok = isfinite(2.f * ord_dec(bounds[6]) * 1.00390625f);
+    for (int c = 0; c < 3; ++c) {
+        const float lo = -ord_dec(bounds[c]), hi = ord_dec(bounds[3 + c]);
+        ok = ok && isfinite(lo) && isfinite(hi) && hi >= lo;
+    }
+    return ok;
+}
+
+// Without a result: an addition whose result is dropped waits for the one before it.
 __device__ __forceinline__ void cluster_max(unsigned addr, unsigned v)
 {
     asm volatile("red.shared::cluster.max.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
+__device__ __forceinline__ void cluster_count(unsigned addr, int v)
+{
+    asm volatile("red.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 
-// Sphere sp of a pill of group grp into the box table (six words as in
-// merge_bounds_to); the lanes `act` call it together, one addition per group.
-__device__ __forceinline__ void box_add(unsigned *box, unsigned act, int grp, float4 sp)
+// A group's box in the table: the corners as unsigned numbers that order as the
+// floats do (ord_enc), the low one inverted so that both grow with the box; zero is
+// the empty box, which meets none.
+struct __align__(16) GroupBox {
+    unsigned lo[4], hi[4];  // the fourth entries only align
+};
+
+// Sphere sp of a pill of group grp into the box table; the lanes `act` call it
+// together, one addition per group.
+__device__ __forceinline__ void box_add(GroupBox *box, unsigned act, int grp, float4 sp)
 {
     const unsigned peers = __match_any_sync(act, grp);
     const float r = cull_reach(sp);
     const bool in = isfinite(sp.x + sp.y + sp.z + r);  // no pair has a sphere that is not
     const float c[3] = {sp.x, sp.y, sp.z};
-    unsigned w[6];
+    unsigned lo[3], hi[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        w[k] = __reduce_max_sync(peers, in ? ord_enc(r - c[k]) : 0u);
-        w[3 + k] = __reduce_max_sync(peers, in ? ord_enc(c[k] + r) : 0u);
+        lo[k] = __reduce_max_sync(peers, in ? ~ord_enc(c[k] - r) : 0u);
+        hi[k] = __reduce_max_sync(peers, in ? ord_enc(c[k] + r) : 0u);
     }
     if ((threadIdx.x & 31) == __ffs(peers) - 1)
 #pragma unroll
-        for (int k = 0; k < 6; ++k) atomicMax(box + 6 * grp + k, w[k]);
+        for (int k = 0; k < 3; ++k) {
+            atomicMax(&box[grp].lo[k], lo[k]);
+            atomicMax(&box[grp].hi[k], hi[k]);
+        }
 }
 
 // The box around group a's meetings with the other groups' boxes, by one warp,
-// written to hot (as floats: low, high; empty: low above high).
-__device__ __forceinline__ void hot_box(const unsigned *box, int groups, int a, float *hot, int lane)
+// written to hot as floats (empty: low above high).
+__device__ __forceinline__ void hot_box(const GroupBox *box, int groups, int a, GroupBox *hot, int lane)
 {
-    float lo[3], hi[3], hl[3] = {INFINITY, INFINITY, INFINITY}, hh[3] = {-INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        lo[k] = -ord_dec(box[6 * a + k]);
-        hi[k] = ord_dec(box[6 * a + 3 + k]);
-    }
+    const uint4 *tab = reinterpret_cast<const uint4 *>(box);
+    const uint4 al = tab[2 * a], ah = tab[2 * a + 1];
+    float hl[3] = {INFINITY, INFINITY, INFINITY}, hh[3] = {-INFINITY, -INFINITY, -INFINITY};
+    bool any = false;
     for (int b = lane; b < groups; b += 32) {
-        if (b == a || box[6 * b] == 0u) continue;
-        float l[3], h[3];
-        bool meet = true;
+        const uint4 bl = tab[2 * b], bh = tab[2 * b + 1];
+        if (b == a || ~al.x > bh.x || ~al.y > bh.y || ~al.z > bh.z || ~bl.x > ah.x || ~bl.y > ah.y || ~bl.z > ah.z)
+            continue;
+        any = true;
+        const unsigned l[3] = {~min(al.x, bl.x), ~min(al.y, bl.y), ~min(al.z, bl.z)};
+        const unsigned h[3] = {min(ah.x, bh.x), min(ah.y, bh.y), min(ah.z, bh.z)};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            l[k] = fmaxf(lo[k], -ord_dec(box[6 * b + k]));
-            h[k] = fminf(hi[k], ord_dec(box[6 * b + 3 + k]));
-            meet = meet && l[k] <= h[k];
+            hl[k] = fminf(hl[k], ord_dec(l[k]));
+            hh[k] = fmaxf(hh[k], ord_dec(h[k]));
         }
-        if (meet)
+    }
+    if (__any_sync(0xffffffffu, any))
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                hl[k] = fminf(hl[k], l[k]);
-                hh[k] = fmaxf(hh[k], h[k]);
+                hl[k] = fminf(hl[k], __shfl_xor_sync(0xffffffffu, hl[k], o));
+                hh[k] = fmaxf(hh[k], __shfl_xor_sync(0xffffffffu, hh[k], o));
             }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            hl[k] = fminf(hl[k], __shfl_xor_sync(0xffffffffu, hl[k], o));
-            hh[k] = fmaxf(hh[k], __shfl_xor_sync(0xffffffffu, hh[k], o));
-        }
     if (lane == 0)
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            hot[k] = hl[k];
-            hot[3 + k] = hh[k];
+            hot->lo[k] = __float_as_uint(hl[k]);
+            hot->hi[k] = __float_as_uint(hh[k]);
         }
 }
 
@@ -360,13 +390,16 @@ __global__ void __launch_bounds__(kGridThreads, 2)
     __shared__ unsigned int s_all[kGridClusterMax][8];  // the CTAs' bounds
     __shared__ unsigned int s_all_kept[kGridClusterMax][8];
     __shared__ int s_tot[kGridClusterMax];              // the ranges' totals
+    __shared__ int s_stay;                              // this CTA's pills that stay
+    __shared__ int s_hist[kRadBins + 33], s_hist_all[kRadBins];  // radii, for the cut (see choose_cut)
     __shared__ int ws[33];
     extern __shared__ __align__(16) unsigned char s_dyn[];
     float4 *s_sph = reinterpret_cast<float4 *>(s_dyn);
     int *s_cell = reinterpret_cast<int *>(s_sph + slice_cap);
     int *s_place = s_cell + slice_cap;
     int *s_count = s_place + slice_cap;
-    unsigned *s_own = reinterpret_cast<unsigned *>(s_count + cells_cap), *s_box = s_own + 6 * groups_cap;
+    GroupBox *s_own = reinterpret_cast<GroupBox *>(s_count + cells_cap), *s_box = s_own + groups_cap;
+    unsigned *own_words = reinterpret_cast<unsigned *>(s_own), *box_words = reinterpret_cast<unsigned *>(s_box);
     int local, nblk;
     batch_scene(A, K_GRID, sb, local, nblk);
     const Params &P = sb.P;
@@ -377,8 +410,10 @@ __global__ void __launch_bounds__(kGridThreads, 2)
     // before the predecessor has finished: what does not depend on the state
     const int groups = P.n_groups <= groups_cap ? P.n_groups : 0;  // 0: every pill stays
     if (t < 8) s_bounds[t] = s_kept[t] = 0u;
+    if (t == 0) s_stay = 0;
     for (int c = t; c < cells_cap; c += bd) s_count[c] = 0;
-    for (int c = t; c < 6 * groups; c += bd) s_own[c] = s_box[c] = 0u;
+    for (int c = t; c < kRadBins; c += bd) s_hist[c] = s_hist_all[c] = 0;
+    for (int c = t; c < 8 * groups; c += bd) own_words[c] = box_words[c] = 0u;
     for (int i = t; i < n; i += bd) {
         s_cell[i] = P.seg_v0[g0 + i];
         s_place[i] = P.seg_group[g0 + i];
@@ -412,7 +447,10 @@ __global__ void __launch_bounds__(kGridThreads, 2)
                 if (i >= n) continue;
                 const float4 sp = pill_sphere(xa[k], ra[k], xb[k], rb[k]);
                 s_sph[i] = sp;
-                if (groups) box_add(s_own, act, s_place[i], sp);
+                if (groups)
+                    box_add(s_own, act, s_place[i], sp);
+                else
+                    hist_add(s_hist, act, sp.w);
                 mn[0] = fminf(mn[0], sp.x); mn[1] = fminf(mn[1], sp.y); mn[2] = fminf(mn[2], sp.z);
                 mx[0] = fmaxf(mx[0], sp.x); mx[1] = fmaxf(mx[1], sp.y); mx[2] = fmaxf(mx[2], sp.z);
                 mr = fmaxf(mr, sp.w);
@@ -423,10 +461,17 @@ __global__ void __launch_bounds__(kGridThreads, 2)
     __syncthreads();
     cluster_wait();  // every CTA of the cluster has started
     for (int k = t; k < 8 * (int)ctas; k += bd) cluster_store(in_cta(&s_all[rank][k & 7], k >> 3), s_bounds[k & 7]);
-    for (int k = t; k < 6 * groups; k += bd)
-        if (s_own[k])
-            for (unsigned r = 0; r < ctas; ++r) cluster_max(in_cta(s_box + k, r), s_own[k]);
-    cluster_sync();  // bounds and boxes exchanged
+    for (int k = t; k < 8 * groups; k += bd)
+        if (own_words[k])
+            for (unsigned r = 0; r < ctas; ++r) cluster_max(in_cta(box_words + k, r), own_words[k]);
+    auto share_hist = [&]() {
+        for (int k = t; k < kRadBins; k += bd)
+            if (s_hist[k])
+                for (unsigned r = 0; r < ctas; ++r) cluster_count(in_cta(s_hist_all + k, r), s_hist[k]);
+    };
+    if (!groups) share_hist();
+    if (rank == 0 && t == 0) P.bp_hist[kRadBins] = 0;  // oversized pills listed
+    cluster_sync();  // bounds and boxes, or bounds and histogram, exchanged
     if (t < 8) {
         unsigned int m = 0u;
         for (unsigned r = 0; r < ctas; ++r) m = max(m, s_all[r][t]);
@@ -439,16 +484,28 @@ __global__ void __launch_bounds__(kGridThreads, 2)
         // the groups of this CTA's pills: their meetings with the others, then the pills that reach them
         const int lane = t & 31;
         for (int a = t >> 5; a < groups; a += bd >> 5)
-            if (s_own[6 * a]) hot_box(s_box, groups, a, reinterpret_cast<float *>(s_own + 6 * a), lane);
+            if (s_own[a].hi[0]) hot_box(s_box, groups, a, s_own + a, lane);
         __syncthreads();
         float kn[3] = {INFINITY, INFINITY, INFINITY}, kx[3] = {-INFINITY, -INFINITY, -INFINITY}, kr = 0.f;
-        for (int i = t; i < n; i += bd) {
-            const float4 sp = s_sph[i];
-            const float r = cull_reach(sp), *hot = reinterpret_cast<const float *>(s_own + 6 * s_place[i]);
-            const bool stays = sp.x - r <= hot[3] && sp.y - r <= hot[4] && sp.z - r <= hot[5] && sp.x + r >= hot[0] &&
-                               sp.y + r >= hot[1] && sp.z + r >= hot[2];
-            s_cell[i] = stays ? 0 : -1;
+        for (int base = 0; base < n; base += bd) {
+            const int i = base + t;
+            bool stays = false;
+            float4 sp;
+            if (i < n) {
+                sp = s_sph[i];
+                const float r = cull_reach(sp);
+                const GroupBox &hot = s_own[s_place[i]];
+                const float4 l = *reinterpret_cast<const float4 *>(hot.lo), h = *reinterpret_cast<const float4 *>(hot.hi);
+                stays = sp.x - r <= h.x && sp.y - r <= h.y && sp.z - r <= h.z && sp.x + r >= l.x && sp.y + r >= l.y &&
+                        sp.z + r >= l.z;
+                s_cell[i] = stays ? 0 : -1;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, stays);
+            int first = 0;
+            if (lane == 0 && m) first = atomicAdd(&s_stay, __popc(m));
+            first = __shfl_sync(0xffffffffu, first, 0);
             if (!stays) continue;
+            s_place[i] = first + __popc(m & ((1u << lane) - 1u));  // among this CTA's
             kn[0] = fminf(kn[0], sp.x); kn[1] = fminf(kn[1], sp.y); kn[2] = fminf(kn[2], sp.z);
             kx[0] = fmaxf(kx[0], sp.x); kx[1] = fmaxf(kx[1], sp.y); kx[2] = fmaxf(kx[2], sp.z);
             kr = fmaxf(kr, fabsf(sp.w));
@@ -456,22 +513,61 @@ __global__ void __launch_bounds__(kGridThreads, 2)
         __syncwarp();
         merge_bounds_to(s_kept, kn, kx, kr);
         __syncthreads();
-        for (int k = t; k < 8 * (int)ctas; k += bd)
-            cluster_store(in_cta(&s_all_kept[rank][k & 7], k >> 3), s_kept[k & 7]);
+        if (t < 8 * (int)ctas)
+            cluster_store(in_cta(&s_all_kept[rank][t & 7], t >> 3), (t & 7) == 7 ? (unsigned)s_stay : s_kept[t & 7]);
         cluster_sync();
-        if (t < 8) {
+        ok = finite_bounds(s_bounds);  // of all pills, as without the cull
+        int total = 0, before = 0;
+        for (unsigned r = 0; r < ctas; ++r) {
+            if (r == rank) before = total;
+            total += (int)s_all_kept[r][7];
+        }
+        if (total <= kGridFew) {  // few stay: one cell of all, every pair tested
+            for (int i = t; i < n; i += bd)
+                if (s_cell[i] >= 0) {
+                    const int pos = before + s_place[i];
+                    P.cell_pills[pos] = g0 + i;
+                    P.cell_sph[pos] = s_sph[i];
+                    P.cell_grp[pos] = P.seg_group[g0 + i];
+                }
+            if (rank == 0 && t == 0) {
+                Grid G = {};
+                for (int c = 0; c < 3; ++c) G.dim[c] = 1;
+                G.b_cut = kRadBins - 1;
+                G.pad = total == 0 || !ok;
+                *P.grid = G;
+                *P.npairs = 0;
+                P.cell_start[0] = 0;
+                P.cell_start[1] = total;
+                if (!ok) atomicOr(P.err, ERR_NONFINITE);
+            }
+            return;
+        }
+        if (t < 7) {
             unsigned int m = 0u;
             for (unsigned r = 0; r < ctas; ++r) m = max(m, s_all_kept[r][t]);
             s_kept[t] = m;
         }
+        for (int base = 0; base < n; base += bd) {
+            const bool in = base + t < n && s_cell[base + t] >= 0;
+            const unsigned act = __ballot_sync(0xffffffffu, in);
+            if (in) hist_add(s_hist, act, s_sph[base + t].w);
+        }
         __syncthreads();
-        make_grid_from(s_bounds, P.table, ok);  // ok: of all pills, as without the cull
-        bool some;
-        G = make_grid_from(s_kept, P.table, some);
-        if (!ok) G.pad = 1;
-    } else {
-        G = make_grid_from(s_bounds, P.table, ok);
+        share_hist();
+        cluster_sync();
     }
+    {
+        const unsigned *bounds = groups ? s_kept : s_bounds;
+        float r_cut;
+        const int b_cut =
+            choose_cut<kRadBins / kGridThreads>(s_hist_all, P.big_cap, 16, ord_dec(bounds[6]), s_hist, &r_cut);
+        bool some;
+        G = make_grid_from(bounds, P.table, some, r_cut, b_cut);
+        if (!groups) ok = some;
+        if (!ok) G.pad = 1;
+    }
+    const unsigned int big = big_threshold(G.b_cut);
     const int cells = (int)min((long long)G.dim[0] * G.dim[1] * G.dim[2], (long long)P.table);
     int sh = 5;  // cells per CTA: 2^sh, at most cells_cap (the table holds at most cells_cap x ctas cells)
     while (((int)ctas << sh) < cells) ++sh;
@@ -480,11 +576,29 @@ __global__ void __launch_bounds__(kGridThreads, 2)
         *P.npairs = 0;
         if (!ok) atomicOr(P.err, ERR_NONFINITE);
     }
-    for (int i = t; i < n; i += bd) {
-        if (groups && s_cell[i] < 0) continue;
-        const int cell = bp_cell(G, s_sph[i]);
-        s_cell[i] = cell;
-        s_place[i] = cluster_add(in_cta(s_count + (cell & ((1 << sh) - 1)), cell >> sh), 1);
+    for (int base = 0; base < n; base += 4 * bd) {  // four additions under way per thread
+        int cell[4], place[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = base + k * bd + t;
+            cell[k] = -1;
+            if (i >= n || (groups && s_cell[i] < 0)) continue;
+            const float4 sp = s_sph[i];
+            if (__float_as_uint(sp.w) > big) {
+                const int slot = atomicAdd(P.bp_hist + kRadBins, 1);
+                if (slot < P.big_cap) P.big_list[slot] = g0 + i;
+                P.spheres[g0 + i] = sp;
+            }
+            cell[k] = bp_cell(G, sp);
+            place[k] = cluster_add(in_cta(s_count + (cell[k] & ((1 << sh) - 1)), cell[k] >> sh), 1);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = base + k * bd + t;
+            if (cell[k] < 0) continue;
+            s_cell[i] = cell[k];
+            s_place[i] = place[k];
+        }
     }
     cluster_sync();  // counts complete
     // exclusive scan of this CTA's cells, warp-strided over consecutive cells
@@ -532,13 +646,25 @@ __global__ void __launch_bounds__(kGridThreads, 2)
         const int *seg_group = P.seg_group;
         int *cell_pills = P.cell_pills, *cell_grp = P.cell_grp;
         float4 *cell_sph = P.cell_sph;
-        for (int i = t; i < n; i += bd) {
-            const int cell = s_cell[i], r = cell >> sh;
-            if (cell < 0) continue;
-            const int pos = s_tot[r] + cluster_load(in_cta(s_count + (cell & ((1 << sh) - 1)), r)) + s_place[i];
-            cell_pills[pos] = g0 + i;
-            cell_sph[pos] = s_sph[i];
-            cell_grp[pos] = seg_group[g0 + i];
+        for (int base = 0; base < n; base += 4 * bd) {
+            int pos[4], grp[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = base + k * bd + t, cell = i < n ? s_cell[i] : -1, r = cell >> sh;
+                pos[k] = -1;
+                if (cell < 0) continue;
+                pos[k] = cluster_load(in_cta(s_count + (cell & ((1 << sh) - 1)), r));
+                grp[k] = seg_group[g0 + i];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = base + k * bd + t;
+                if (pos[k] < 0) continue;
+                const int at = s_tot[s_cell[i] >> sh] + pos[k] + s_place[i];
+                cell_pills[at] = g0 + i;
+                cell_sph[at] = s_sph[i];
+                cell_grp[at] = grp[k];
+            }
         }
     }
     {
@@ -579,10 +705,17 @@ __global__ void __launch_bounds__(256, 2) batch_rod_kernel(BatchArgs A, int firs
     __shared__ BatchScene sb;
     extern __shared__ float4 smem[];
     int local, nblk;
-    batch_enter(A, K_ROD, sb, local, nblk);
-    // read after rod_item's first barrier
+    batch_scene(A, K_ROD, sb, local, nblk);
+    RodStage S;
+    rod_stage_rest(sb.P, local, first != 0, S);
+    // after a contact pass: the state and the pair count are those it started from
+    if (!first) rod_stage_state(sb.P, S, smem);
+    // read after rod_run's first barrier
     if (threadIdx.x == 0 && !packs_used(sb.P, first != 0)) sb.P.XW = nullptr;
-    rod_item(sb.P, local, first != 0, apply != 0, smem);
+    pdl_wait();
+    pdl_trigger();
+    if (first) rod_stage_state(sb.P, S, smem);
+    rod_run(sb.P, S, apply != 0, smem);
 }
 
 // Every substep of the frame (no contacts).
@@ -602,13 +735,16 @@ __global__ void __launch_bounds__(kElemThreads, 4) batch_contact_kernel(BatchArg
     __shared__ BatchScene sb;
     __shared__ QueuedPair queue[kElemThreads / 32][64];
     int local, nblk;
-    batch_enter(A, K_CONTACT, sb, local, nblk);
+    batch_scene(A, K_CONTACT, sb, local, nblk);
     Params &P = sb.P;
+    if (first) pdl_wait();  // the pair search is finished before any later pass's sweep begins
+    const int np_all = sb.pills ? *P.npairs : 0;
     if (threadIdx.x == 0 && !packs_used(P, first != 0)) {
         P.XW = nullptr;
         P.PB = nullptr;
     }
-    const int np_all = sb.pills ? *P.npairs : 0;
+    if (!first) pdl_wait();
+    pdl_trigger();
     __syncthreads();
     const int np = min(np_all, P.max_pairs);
     if (local == 0 && threadIdx.x == 0 && np_all > P.max_pairs) atomicOr(P.err, ERR_OVERFLOW);
@@ -646,14 +782,22 @@ __global__ void __launch_bounds__(kElemThreads) batch_advance_kernel(BatchArgs A
 {
     __shared__ BatchScene sb;
     int local, nblk;
-    batch_enter(A, K_ELEM, sb, local, nblk);
+    batch_scene(A, K_ELEM, sb, local, nblk);
     const Params &P = sb.P;
+    const int i = local * blockDim.x + threadIdx.x, nv = P.nv;
+    const bool fin = finish_prev != 0, vertex = i < nv, segment = !vertex && i < nv + P.ns, world = sb.pills != 0;
+    // loaded while the previous substep's last contact pass still runs, unless shape
+    // matching or the warm start runs in between
+    const bool state = fin && P.n_xs == 0;
+    AdvanceVertex V;
+    AdvanceSegment G;
+    if (vertex) advance_vertex_load(P, i, fin, state, tau, world, V);
+    if (segment) advance_segment_load(P, i - nv, fin, state, G);
+    pdl_wait();
+    pdl_trigger();
     if (sb.pills && local == 0 && threadIdx.x < 8) P.bounds[threadIdx.x] = 0u;
-    const int i = local * blockDim.x + threadIdx.x;
-    if (i < P.nv)
-        advance_vertex_at(P, i, finish_prev != 0, tau, sb.pills != 0);
-    else if (i < P.nv + P.ns)
-        advance_segment_at(P, i - P.nv, finish_prev != 0);
+    if (vertex) advance_vertex_at(P, i, fin, state, world, V);
+    if (segment) advance_segment_at(P, i - nv, fin, state, G);
 }
 
 // Warm start from the bones before the frame's first substep (scenes with a warm-start table).
@@ -764,12 +908,22 @@ int grid_cluster(int scenes, int max_ns, int max_table)
     return c;
 }
 
+// CTAs for a scene's `part` of the group's `all` pills: what it could use, `want`,
+// within its share of the four CTAs an SM holds.  A CTA without work still costs its
+// start: 64 scenes with 1,738 CTAs each for the search and the passes, most of
+// them idle, took 3.00 ms a frame, with 577 2.86.
+int resident_share(int want, int part, long long all)
+{
+    const long long most = 4LL * device_sm_count() * part / std::max(all, 1LL);
+    return (int)std::max(1LL, std::min((long long)want, most));
+}
+
 // Groups of few pills do not fill the GPU with a thread per pill: several lanes
 // search a pill's neighbours (200 muscles, 6,910 pills, before the cull: 1,955 us
 // for two frames with one lane, 1,505 with two, 1,305 with four, 1,200 with eight;
 // strands and many scenes are fastest with one to four), and a contact CTA covers
 // fewer pills.
-constexpr int kSmallGroup = 16384, kEmitLanesSmall = 4, kContactPillsSmall = 64;
+constexpr int kSmallGroup = 20000, kEmitLanesSmall = 4, kContactPillsSmall = 64;
 constexpr int kMeshPerThread = 16;  // kLbsBatch vertices per round, 16 / kLbsBatch rounds
 
 size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -836,7 +990,8 @@ struct Fork {
 // Launch shape of one sequence: blocks per kernel kind over all its scenes.
 struct Shape {
     int tot[K_KINDS] = {};
-    bool small = false;  // few pills (kSmallGroup)
+    bool small = false;        // few pills (kSmallGroup)
+    long long all_pills = 0;   // segments of the group's scenes
     int threads = 0, smem = 16;
     bool cp = false, fused_grid = true;
     int cluster = kGridClusterMax, cells_cap = 32, slice_cap = 32, groups_cap = 0;  // grid build: CTAs per scene, shared memory
@@ -876,13 +1031,16 @@ void fill_scene(BatchScene &b, int cnt[K_KINDS], viper_scene *s, const viper_bat
     const int nv = s->nv, ns = s->ns;
     cnt[K_ELEM] = cdiv(nv + ns, kElemThreads);
     cnt[K_PILL] = b.pills ? cdiv(ns, kElemThreads) : 0;
-    cnt[K_EMIT] = b.pills ? cdiv((long long)ns * (sh.small ? kEmitLanesSmall : 1), 32 * kEmitWarpsB) : 0;
+    // pair search and contact pass: grid-stride over the scene's pills and pairs, so no
+    // more CTAs than stay resident, shared out by size (see resident_share)
+    const long long want_emit = (long long)ns * (sh.small ? kEmitLanesSmall : 1);
+    cnt[K_EMIT] = b.pills ? resident_share(cdiv(want_emit, 32 * kEmitWarpsB), ns, sh.all_pills) : 0;
     cnt[K_SCAN] = b.pills ? 1 : 0;
     cnt[K_GRID] = b.pills ? sh.cluster : 0;
     cnt[K_ROD] = s->n_items;
-    cnt[K_CONTACT] = cp ? std::min(4 * device_sm_count(),
-                                   std::max(1, cdiv(ns + (s->n_planes > 0 ? nv : 0), sh.small ? kContactPillsSmall : kElemThreads)))
-                        : 0;
+    const int touch = ns + (s->n_planes > 0 ? nv : 0);
+    cnt[K_CONTACT] =
+        cp ? resident_share(cdiv(touch, sh.small ? kContactPillsSmall : kElemThreads), ns, sh.all_pills) : 0;
     cnt[K_END] = it.n_mesh > 0 ? std::max(1, cdiv(ns, kElemThreads)) : 1;
     cnt[K_MESH] = cdiv(it.n_mesh, kElemThreads * kMeshPerThread);
     cnt[K_BUNDLE] = cp ? cdiv(s->P.n_xs, kElemThreads / 32) : 0;
@@ -896,7 +1054,7 @@ void shape_add(Shape &sh, const viper_scene *s, bool cp)
     if (cp && (s->flags & VIPER_FLAG_CONTACTS)) {
         if (s->ns > kGridMaxPills) sh.fused_grid = false;
         sh.cells_cap = std::max(sh.cells_cap, s->P.table / sh.cluster);
-        sh.slice_cap = std::max(sh.slice_cap, cdiv(s->ns, sh.cluster));
+        sh.slice_cap = std::max(sh.slice_cap, cdiv(s->ns, 4 * sh.cluster) * 4);
         if (s->P.n_groups <= kGridGroupsMax) sh.groups_cap = std::max(sh.groups_cap, s->P.n_groups);
     }
     sh.threads = s->block_threads;
@@ -953,15 +1111,18 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
         for (int k = 0; k < substeps; ++k) {
             const float tau = (float)((double)(k + 1) / substeps);  // as the one-scene path
             if (forked) {
-                // advance | [grid, pair search] beside [first sweep] | contact ...
+                // advance | [grid, pair search] beside [first sweep] | contact ...; the grid and
+                // the pair search take longer than the sweep, so they follow on the main
+                // stream, where their prologues overlap what is before them
                 go(PROF_ELEM, [&] { launch(batch_advance_kernel, tot[K_ELEM], kElemThreads, 0, st, A, k > 0 ? 1 : 0, tau); });
                 if (cudaEventRecord(fork->ev_fork, st) != cudaSuccess ||
                     cudaStreamWaitEvent(fork->side, fork->ev_fork, 0) != cudaSuccess)
                     return -1;
-                broadphase(fork->side);
-                if (cudaEventRecord(fork->ev_join, fork->side) != cudaSuccess) return -1;
-                go(PROF_ROD, [&] { launch(batch_rod_kernel, tot[K_ROD], threads, smem, st, A, 1, 0); });
-                if (cudaStreamWaitEvent(st, fork->ev_join, 0) != cudaSuccess) return -1;
+                broadphase(st);
+                go(PROF_ROD, [&] { launch(batch_rod_kernel, tot[K_ROD], threads, smem, fork->side, A, 1, 0); });
+                if (cudaEventRecord(fork->ev_join, fork->side) != cudaSuccess ||
+                    cudaStreamWaitEvent(st, fork->ev_join, 0) != cudaSuccess)
+                    return -1;
             } else {
                 go(PROF_ROD, [&] { launch(batch_rod_first_kernel, tot[K_ROD], threads, smem, st, A, k > 0 ? 1 : 0, tau); });
                 broadphase(st);
@@ -1029,6 +1190,7 @@ int run_group(viper_batch *B, const viper_batch_item *items, const std::vector<i
         }
     sh.cluster = grid_cluster(pill_scenes, max_ns, max_table);
     sh.small = group_pills <= kSmallGroup;
+    for (int i : idx) sh.all_pills += items[i].scene->ns;
     for (int c = 0; c < K_KINDS; ++c) off[c * (n + 1)] = 0;
     for (int k = 0; k < n; ++k) {
         const viper_batch_item &it = items[idx[k]];
@@ -1092,6 +1254,7 @@ int self_batch_capture(viper_scene *s, float dt, int substeps, int iterations, c
     int cnt[K_KINDS];
     Shape sh;
     sh.small = s->ns <= kSmallGroup;
+    sh.all_pills = s->ns;
     sh.cluster = grid_cluster(1, s->ns, s->P.table);
     fill_scene(*b, cnt, s, it, (double)dt / substeps, cp, sh);  // bones: the scene's own target pose
     shape_add(sh, s, cp);

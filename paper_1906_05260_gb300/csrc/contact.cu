@@ -27,7 +27,7 @@ namespace viper {
 
 // Bounding spheres, their bounds and the histogram of their radii (the
 // kBoundsWords bounds words are zeroed before; see merge_bounds, choose_cut).
-constexpr int kBpThreads = 256;  // choose_cut takes two histogram bins per thread
+constexpr int kBpThreads = 256;
 __global__ void __launch_bounds__(kBpThreads) bp_bounds_kernel(Params P)
 {
     __shared__ int hist[kRadBins];
@@ -45,10 +45,7 @@ __global__ void __launch_bounds__(kBpThreads) bp_bounds_kernel(Params P)
         mn[0] = fminf(mn[0], sp.x); mn[1] = fminf(mn[1], sp.y); mn[2] = fminf(mn[2], sp.z);
         mx[0] = fmaxf(mx[0], sp.x); mx[1] = fmaxf(mx[1], sp.y); mx[2] = fmaxf(mx[2], sp.z);
         mr = fmaxf(mr, sp.w);
-        // most pills of a scene share a few bins: one addition per bin and warp
-        const int bin = rad_bin(sp.w);
-        const unsigned peers = __match_any_sync(in, bin);
-        if (lane == __ffs(peers) - 1) atomicAdd(hist + bin, __popc(peers));
+        hist_add(hist, in, sp.w);
     }
     __syncwarp();
     merge_bounds_to(s_bounds, mn, mx, mr);
@@ -66,7 +63,7 @@ __global__ void __launch_bounds__(kBpThreads) bp_count_kernel(Params P)
 {
     __shared__ int sh[kRadBins + 33];
     float r_cut;
-    const int b_cut = choose_cut(P.bp_hist, P.big_cap, ord_dec(P.bounds[6]), sh, &r_cut);
+    const int b_cut = choose_cut<kRadBins / kBpThreads>(P.bp_hist, P.big_cap, 1, ord_dec(P.bounds[6]), sh, &r_cut);
     bool ok;
     const Grid G = make_grid_from(P.bounds, P.table, ok, r_cut, b_cut);
     if (blockIdx.x == 0 && threadIdx.x == 0) {

@@ -217,42 +217,77 @@ __device__ __forceinline__ void predict_segment_at(const Params &P, int g, bool 
     }
 }
 
-// The start of a substep for vertex v without its first sweep: with
+// The start of a substep for vertex v (segment g) without its first sweep: with
 // `finish_prev`, the previous substep's pending contact corrections and
 // velocity update; then the prediction (Sec. 6) at bone fraction tau, the
 // substep's start state in Xp, the predicted world position for the
 // broadphase when `world`, and cleared half-plane multipliers (as the first
-// sweep kernel does before its sweep).
-__device__ __forceinline__ void advance_vertex_at(const Params &P, int v, bool finish_prev, float tau, bool world)
+// sweep kernel does before its sweep).  advance_*_load reads what the last
+// contact pass does not change (`state`: the positions and frames too, which
+// shape matching and the warm start do change), and works out a pinned vertex's
+// target; advance_*_at does the rest.
+struct AdvanceVertex {
+    float4 x, xp, vel, rv1, o;
+    V3 pin;
+};
+__device__ __forceinline__ void advance_vertex_load(const Params &P, int v, bool finish_prev, bool state, float tau,
+                                                    bool world, AdvanceVertex &A)
 {
-    float4 x = P.X[v], vel;
+    A.rv1 = P.RV1[v];
+    if (state) A.x = P.X[v];
+    if (finish_prev)
+        A.xp = P.Xp[v];
+    else
+        A.vel = P.V[v];
+    if (world) A.o = P.rod_origin[P.rod_of_v[v]];
+    if (A.rv1.x < 0.f) A.pin = pin_target(P, __float2int_rn(-A.rv1.x) - 1, tau);
+}
+
+__device__ __forceinline__ void advance_vertex_at(const Params &P, int v, bool finish_prev, bool state, bool world,
+                                                  AdvanceVertex &A)
+{
+    float4 x = state ? A.x : P.X[v];
+    float4 vel = A.vel;
     if (finish_prev) {
         x = apply_pending(P, v, x);
-        const float4 xp = P.Xp[v];
+        const float4 xp = A.xp;
         vel = make_float4((x.x - xp.x) * P.inv_h, (x.y - xp.y) * P.inv_h, (x.z - xp.z) * P.inv_h,
                           (x.w - xp.w) * P.inv_h);
         check_finite(P, x);
         P.V[v] = vel;
-    } else {
-        vel = P.V[v];
     }
     P.Xp[v] = x;
-    x = predict_vertex(P, x, vel, P.RV1[v], tau);
-    if (world) P.Xpred[v] = to_world(P, v, x);
+    if (A.rv1.x < 0.f)
+        x = make_float4(A.pin.x, A.pin.y, A.pin.z, x.w + P.h * vel.w);
+    else
+        x = predict_vertex(P, x, vel, A.rv1, 0.f);
+    if (world) P.Xpred[v] = make_float4(__fadd_rn(x.x, A.o.x), __fadd_rn(x.y, A.o.y), __fadd_rn(x.z, A.o.z), x.w);
     for (int k = 0; k < P.n_planes; ++k) P.lam_plane[(size_t)v * P.n_planes + k] = 0.f;
     P.X[v] = x;
 }
 
-__device__ __forceinline__ void advance_segment_at(const Params &P, int g, bool finish_prev)
+struct AdvanceSegment {
+    float4 q, qp, w;
+};
+__device__ __forceinline__ void advance_segment_load(const Params &P, int g, bool finish_prev, bool state,
+                                                     AdvanceSegment &A)
 {
-    const float4 q = P.Q[g];
-    float4 w;
+    if (state) A.q = P.Q[g];
+    if (finish_prev)
+        A.qp = P.Qp[g];
+    else
+        A.w = P.W[g];
+}
+
+__device__ __forceinline__ void advance_segment_at(const Params &P, int g, bool finish_prev, bool state,
+                                                   const AdvanceSegment &A)
+{
+    const float4 q = state ? A.q : P.Q[g];
+    float4 w = A.w;
     if (finish_prev) {
         check_finite(P, q);
-        w = omega_of(P, q, P.Qp[g]);
+        w = omega_of(P, q, A.qp);
         P.W[g] = w;
-    } else {
-        w = P.W[g];
     }
     P.Qp[g] = q;
     P.Q[g] = predict_quat(P, q, w);
@@ -605,36 +640,50 @@ __device__ __forceinline__ void sweep_any(const Params &P, SmemRod sX, SmemRod s
     }
 }
 
-// One sweep of one work item between contact passes: a CTA stages the item's
-// float4 state in shared memory with coalesced loads (adding the pending contact
-// corrections when `apply`), runs a sweep with each thread's constraints held in
-// registers, and writes the state back.  Item b's slot descriptors and
-// multipliers are entries b * blockDim.x + threadIdx.x.  Every thread of the
-// CTA must call it.
-__device__ __forceinline__ void rod_item(const Params &P, int b, bool first, bool apply, float4 *smem)
+// One sweep of one work item between contact passes, in two parts.  rod_stage: a
+// CTA stages the item's float4 state in shared memory with coalesced loads and
+// each thread's rest data and multipliers in registers.  rod_run adds the pending
+// contact corrections when `apply`, runs a sweep and writes the state back.  Item
+// b's slot descriptors and multipliers are entries b * blockDim.x + threadIdx.x.
+// Every thread of the CTA calls both.  A contact pass changes nothing that
+// rod_stage reads, so the sweep after it can stage while the pass still runs.
+struct RodStage {
+    int4 item;
+    int slot;
+    SlotRest R;
+    SlotLam L;
+};
+
+__device__ __forceinline__ void rod_stage_rest(const Params &P, int b, bool first, RodStage &S)
 {
-    const int4 item = P.items[b];
+    S.item = P.items[b];
+    S.slot = b * blockDim.x + threadIdx.x;
+    load_slot(P, S.item, P.slots[S.slot], S.R);
+    if (first)
+        zero_lam(S.L);
+    else
+        lam_load(P, S.slot, S.L);
+}
+
+__device__ __forceinline__ void rod_stage_state(const Params &P, const RodStage &S, float4 *smem)
+{
+    const int4 item = S.item;
     const SmemRod sX = smem_rod(smem, item.y);
     const SmemRod sQ = smem_rod(smem + item.y, item.w);
-
-    for (int i = threadIdx.x; i < item.y; i += blockDim.x) {
-        float4 x = P.X[item.x + i];
-        if (apply) x = apply_pending(P, item.x + i, x);
-        sX[i] = x;
-    }
+    for (int i = threadIdx.x; i < item.y; i += blockDim.x) sX[i] = P.X[item.x + i];
     for (int j = threadIdx.x; j < item.w; j += blockDim.x) sQ[j] = P.Q[item.z + j];
+}
 
-    const int slot = b * blockDim.x + threadIdx.x;
-    SlotRest R;
-    load_slot(P, item, P.slots[slot], R);
-    SlotLam L;
-    if (first)
-        zero_lam(L);
-    else
-        lam_load(P, slot, L);
+__device__ __forceinline__ void rod_run(const Params &P, RodStage &S, bool apply, float4 *smem)
+{
+    const int4 item = S.item;
+    const SmemRod sX = smem_rod(smem, item.y);
+    const SmemRod sQ = smem_rod(smem + item.y, item.w);
+    if (apply)  // to the elements this thread staged
+        for (int i = threadIdx.x; i < item.y; i += blockDim.x) sX[i] = apply_pending(P, item.x + i, sX[i]);
     __syncthreads();
-    sweep_any(P, sX, sQ, R, L, smem + 2 * (item.y + item.w), item);  // Jacobi records behind the state
-    if (R.active) lam_store(P, slot, L);
+    sweep_any(P, sX, sQ, S.R, S.L, smem + 2 * (item.y + item.w), item);  // Jacobi records behind the state
+    if (S.R.active) lam_store(P, S.slot, S.L);
 
     for (int i = threadIdx.x; i < item.y; i += blockDim.x) {
         const int v = item.x + i;
@@ -970,28 +1019,46 @@ __device__ __forceinline__ unsigned int big_threshold(int b_cut)
     return b_cut < kRadBins - 1 ? (((unsigned)b_cut + 1u + kRadBinBase) << 19) - 1u : 0xffffffffu;
 }
 
-// Cut bin from the histogram, by every thread of a 256-thread block (the same
-// result in every block): the smallest b such that bins above b hold at most
-// `cap` pills.  Returns b_cut; *r_cut = the top edge of bin b_cut, or the
-// largest radius when no pill lies above it.  sh: kRadBins + 33 ints of shared memory.
-__device__ __forceinline__ int choose_cut(const int *hist, int cap, float r_max, int *sh, float *r_cut)
+// Cut bin from the histogram, by every thread of a block of kRadBins / PER
+// threads (the same result in every block): the smallest b such that bins above
+// b hold at most `cap` pills, or all / `share` of those counted if that is fewer
+// (a cut that takes half of a few pills out makes cells far below their size).  Returns b_cut; *r_cut = the top edge of bin
+// b_cut, or the largest radius when no pill lies above it.  sh: kRadBins + 33
+// ints of shared memory.
+template <int PER>
+__device__ __forceinline__ int choose_cut(const int *hist, int cap, int share, float r_max, int *sh, float *r_cut)
 {
     int *h = sh, *ws = sh + kRadBins;
-    const int t = threadIdx.x;  // bins 511 - 2t and 510 - 2t (suffix sums from the top)
-    const int b0 = kRadBins - 1 - 2 * t, b1 = b0 - 1;
-    const int h0 = hist[b0], h1 = hist[b1];
-    int tot;
-    const int above = block_excl_scan(h0 + h1, ws, &tot);  // pills in bins > b0
-    h[b0] = above;            // pills in bins > b0
-    h[b1] = above + h0;       // pills in bins > b1
+    const int b0 = kRadBins - 1 - PER * threadIdx.x;  // bins b0, b0 - 1, ... (suffix sums from the top)
+    int n[PER], tot, sum = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) sum += n[j] = hist[b0 - j];
+    int above = block_excl_scan(sum, ws, &tot);  // pills in bins > b0
+    cap = min(cap, tot / share);
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        h[b0 - j] = above;
+        above += n[j];
+    }
     __syncthreads();
     // bins b with (pills above b) <= cap form a top range [b_cut, kRadBins); its size
-    const int n_ok = __syncthreads_count(h[b0] <= cap) + __syncthreads_count(h[b1] <= cap);
+    int n_ok = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) n_ok += __syncthreads_count(h[b0 - j] <= cap);
     const int b_cut = max(kRadBins - n_ok, 0);
     const bool none_above = h[b_cut] == 0;
     __syncthreads();
     *r_cut = none_above ? r_max : rad_bin_top(b_cut);
     return none_above ? kRadBins - 1 : b_cut;
+}
+
+// One more pill of radius R in the histogram; the lanes `act` call it together
+// (most pills of a scene share a few bins: one addition per bin and warp).
+__device__ __forceinline__ void hist_add(int *hist, unsigned act, float R)
+{
+    const int bin = rad_bin(R);
+    const unsigned peers = __match_any_sync(act, bin);
+    if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(hist + bin, __popc(peers));
 }
 
 __device__ __forceinline__ void count_pill(const Params &P, const Grid &G, int g)

@@ -182,7 +182,10 @@ __global__ void bundle_kernel(Params P)
 __global__ void __launch_bounds__(256) rod_kernel(Params P, int first, int apply)
 {
     extern __shared__ float4 smem[];
-    rod_item(P, blockIdx.x, first != 0, apply != 0, smem);
+    RodStage S;
+    rod_stage_rest(P, blockIdx.x, first != 0, S);
+    rod_stage_state(P, S, smem);
+    rod_run(P, S, apply != 0, smem);
 }
 
 __global__ void __launch_bounds__(256) rod_frame_kernel(Params P, int substeps, int n_iter)

@@ -37,6 +37,7 @@ def _scene(seed, rods, verts, spread, groups=None, seg=0.01, far=0.0, thick=1.0)
     dict(seed=6, rods=512, verts=3, spread=0.15), dict(seed=7, rods=513, verts=3, spread=0.15),
     dict(seed=8, rods=700, verts=12, spread=0.3, groups=25, thick=9.0), dict(seed=9, rods=300, verts=20, spread=0.2, far=50.0),
     dict(seed=10, rods=1100, verts=16, spread=0.4, thick=3.0),
+    dict(seed=11, rods=512, verts=81, spread=0.5), dict(seed=12, rods=513, verts=81, spread=0.5),  # 40,960 pills, and more
 ], ids=lambda k: "-".join(f"{a}{b}" for a, b in k.items() if a != "seed"))
 def test_scene_pairs_match_brute_force(kw):
     from paper_1906_05260_gb300 import viper as V
