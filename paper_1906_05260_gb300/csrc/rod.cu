@@ -179,7 +179,12 @@ __global__ void bundle_kernel(Params P)
 }
 
 // ------------------------------------------------------------------ shared-memory rods
-__global__ void __launch_bounds__(256) rod_kernel(Params P, int first, int apply)
+// 96 registers (the compiler would take 123) let five CTAs of 128 threads on an SM
+// instead of four: the sweep waits for its loads (issue slots 37 % used at 16
+// warps an SM).  20,000 falling strands, a frame 3.19 -> 3.04 ms; 80 registers spill
+// and take 3.14.  Alone on the GPU, as the smaller scenes of the one-scene graph
+// run, a CTA gains nothing and pays for the spills: they keep 128.
+__global__ void __maxnreg__(96) rod_kernel(Params P, int first, int apply)
 {
     extern __shared__ float4 smem[];
     RodStage S;
