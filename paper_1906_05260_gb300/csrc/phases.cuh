@@ -1837,13 +1837,6 @@ __device__ __forceinline__ void ld_frame(const float4 *f, float4 &r, float4 &ts)
 // frame is 32 bytes: the relative rotation r = R_j Rbar_j^T as a unit
 // quaternion and (t, s_m) with t = c_m - s_m r cbar_m, so T Tbar^-1 p = s_m r p + t.
 // Frame ids outside [0, ns) contribute nothing and raise the error word.
-// Frame k of a table in shared memory (two 128-bit shared loads).
-__device__ __forceinline__ void ld_frame_shared(const float4 *f, float4 &r, float4 &ts)
-{
-    r = f[0];
-    ts = f[1];
-}
-
 template <bool SHARED>
 __device__ __forceinline__ float4 lbs_blend(float4 p, int4 id, float4 ww, int ns, const float4 *__restrict__ frames,
                                            int *err)
@@ -1857,12 +1850,13 @@ __device__ __forceinline__ float4 lbs_blend(float4 p, int4 id, float4 ww, int ns
             atomicOr(err, ERR_OVERFLOW);
             continue;
         }
-        const float4 *f = frames + kLbsFrame * (size_t)ids[k];
         float4 r, ts;
-        if (SHARED)
-            ld_frame_shared(f, r, ts);
-        else
-            ld_frame(f, r, ts);
+        if (SHARED) {  // a table of rotations, then one of translations (see lbs_gather_smem_kernel)
+            r = frames[ids[k]];
+            ts = frames[ns + ids[k]];
+        } else {
+            ld_frame(frames + kLbsFrame * (size_t)ids[k], r, ts);
+        }
         const V3 y = qrot(r, v3(p.x, p.y, p.z));
         ox += wv[k] * (ts.w * y.x + ts.x);
         oy += wv[k] * (ts.w * y.y + ts.y);
