@@ -580,7 +580,13 @@ void enqueue_frame(viper_scene *s, float dt, int substeps, int iterations)
                 launch_finish(s, s->resident_nv, nv, s->resident_ns, ns, false);
             }
         } else {
-            launch_predict(s, 0, nv, 0, ns, true);
+            // with every rod in the shared-memory sweep the prediction follows the previous
+            // substep's velocity update in one kernel (it clears no streamed rods' multipliers)
+            const bool fused = s->resident_nv == nv && iterations > 0;
+            if (fused)
+                launch_advance(s, k > 0, pills);
+            else
+                launch_predict(s, 0, nv, 0, ns, true);
             // the broadphase only needs the predicted state: run it on a second
             // branch beside the first constraint sweep, join before the first contact pass
             bool forked = false;
@@ -605,7 +611,7 @@ void enqueue_frame(viper_scene *s, float dt, int substeps, int iterations)
                 launch_contacts(s);
             }
             if (iterations > 0) launch_bundles(s);
-            launch_finish(s, 0, nv, 0, ns, iterations > 0);
+            if (!fused || k + 1 == substeps) launch_finish(s, 0, nv, 0, ns, iterations > 0);
         }
     }
     if (s->n_bones > 0) {

@@ -256,6 +256,7 @@ struct ProfScope {
 
 // launchers (all enqueue on s->stream and count kernels in s->launches)
 void launch_predict(viper_scene *s, int v_begin, int v_end, int s_begin, int s_end, bool contact_path);
+void launch_advance(viper_scene *s, bool finish_prev, bool world);
 void launch_finish(viper_scene *s, int v_begin, int v_end, int s_begin, int s_end, bool apply);
 void launch_colour(viper_scene *s, int colour, const int *list, int n);
 void launch_rod_frame(viper_scene *s, int substeps, int n_iter);
