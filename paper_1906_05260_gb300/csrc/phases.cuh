@@ -338,7 +338,12 @@ __device__ __forceinline__ void lam_load(const Params &P, int slot, SlotLam &L)
     const int st = P.slot_stride;
     float t[kSlotLam];
 #pragma unroll
-    for (int k = 0; k < kSlotLam; ++k) t[k] = b[k * st];
+    for (int k = 0; k < kSlotLam - 2; ++k) t[k] = b[k * st];
+    t[22] = t[23] = 0.f;
+    if (P.surface) {
+        t[22] = b[22 * st];
+        t[23] = b[23 * st];
+    }
     L.s0 = make_float4(t[0], t[1], t[2], t[3]);
     L.s1 = make_float4(t[4], t[5], t[6], t[7]);
     L.b1 = make_float4(t[8], t[9], t[10], t[11]);
@@ -359,7 +364,11 @@ __device__ __forceinline__ void lam_store(const Params &P, int slot, const SlotL
                                L.b1.x, L.b1.y, L.b1.z, L.b1.w, L.b2.x, L.b2.y, L.b2.z, L.b2.w,
                                L.x0.x, L.x0.y, L.x1.x, L.x1.y, L.v1, L.v2, L.l1, L.l2};
 #pragma unroll
-    for (int k = 0; k < kSlotLam; ++k) b[k * st] = t[k];
+    for (int k = 0; k < kSlotLam - 2; ++k) b[k * st] = t[k];
+    if (P.surface) {
+        b[22 * st] = t[22];
+        b[23 * st] = t[23];
+    }
 }
 
 

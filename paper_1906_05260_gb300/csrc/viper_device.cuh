@@ -87,10 +87,15 @@ __device__ __forceinline__ V3 qrot(float4 q, V3 v)
     V3 t = 2.f * cross(u, v);
     return v + q.w * t + cross(u, t);
 }
-// q <- normalize(q + 1/2 (d, 0) q)
+// q <- normalize(q + 1/2 (d, 0) q): qmul without the products with the zero, which the
+// compiler has to keep, each rounding where qmul has it
 __device__ __forceinline__ void rotate_by(float4 &q, V3 d)
 {
-    float4 t = qmul(make_float4(d.x, d.y, d.z, 0.f), q);
+    const float4 t =
+        make_float4(__fmaf_rn(-d.z, q.y, __fmaf_rn(d.y, q.z, __fmul_rn(q.w, d.x))),
+                    __fmaf_rn(-d.x, q.z, __fmaf_rn(d.z, q.x, __fmul_rn(q.w, d.y))),
+                    __fmaf_rn(-d.y, q.x, __fmaf_rn(d.x, q.y, __fmul_rn(q.w, d.z))),
+                    __fmaf_rn(-d.z, q.z, __fmaf_rn(-d.y, q.y, __fmul_rn(-d.x, q.x))));
     q = qnormalize(make_float4(q.x + 0.5f * t.x, q.y + 0.5f * t.y, q.z + 0.5f * t.z, q.w + 0.5f * t.w));
 }
 
@@ -330,8 +335,7 @@ __device__ __forceinline__ void rel_frame(RelFrame &f, float4 qa, float4 qb, flo
     f.e = qd3(p);
     V3 pv = {p.x, p.y, p.z};
     // M ez and M e, with M v = p_w v - p_v x v
-    V3 ez = {0.f, 0.f, 1.f};
-    V3 m1 = p.w * ez - cross(pv, ez);
+    V3 m1 = {-p.y, p.x, p.w};
     V3 m2 = p.w * f.e - cross(pv, f.e);
     float c0 = f.da + f.db, c1 = -0.5f * f.da, c2 = -0.5f * f.db;
     f.N[0] = c0 * (1.f - pv.x * pv.x) + c1 * m1.x * m1.x + c2 * m2.x * m2.x;
