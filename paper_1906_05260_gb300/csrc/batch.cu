@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(kGridThreads, 2)
                     hist_add(s_hist, act, sp.w);
                 mn[0] = fminf(mn[0], sp.x); mn[1] = fminf(mn[1], sp.y); mn[2] = fminf(mn[2], sp.z);
                 mx[0] = fmaxf(mx[0], sp.x); mx[1] = fmaxf(mx[1], sp.y); mx[2] = fmaxf(mx[2], sp.z);
-                mr = fmaxf(mr, sp.w);
+                mr = fmaxf(mr, fabsf(sp.w));
             }
         }
     }
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(kGridThreads, 2)
         const int b_cut =
             choose_cut<kRadBins / kGridThreads>(s_hist_all, P.big_cap, 16, ord_dec(bounds[6]), s_hist, &r_cut);
         bool some;
-        G = make_grid_from(bounds, P.table, some, r_cut, b_cut);
+        G = make_grid_from(bounds, P.table, some, r_cut, b_cut, true);
         if (!groups) ok = some;
         if (!ok) G.pad = 1;
     }

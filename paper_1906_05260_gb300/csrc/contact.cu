@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kBpThreads) bp_bounds_kernel(Params P)
         P.spheres[g0 + lane] = sp;
         mn[0] = fminf(mn[0], sp.x); mn[1] = fminf(mn[1], sp.y); mn[2] = fminf(mn[2], sp.z);
         mx[0] = fmaxf(mx[0], sp.x); mx[1] = fmaxf(mx[1], sp.y); mx[2] = fmaxf(mx[2], sp.z);
-        mr = fmaxf(mr, sp.w);
+        mr = fmaxf(mr, fabsf(sp.w));
         hist_add(hist, in, sp.w);
     }
     __syncwarp();
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kBpThreads) bp_count_kernel(Params P)
     float r_cut;
     const int b_cut = choose_cut<kRadBins / kBpThreads>(P.bp_hist, P.big_cap, 1, ord_dec(P.bounds[6]), sh, &r_cut);
     bool ok;
-    const Grid G = make_grid_from(P.bounds, P.table, ok, r_cut, b_cut);
+    const Grid G = make_grid_from(P.bounds, P.table, ok, r_cut, b_cut, true);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *P.grid = G;
         *P.npairs = 0;  // pair cursor of bp_emit_kernel

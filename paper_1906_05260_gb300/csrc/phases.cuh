@@ -854,8 +854,13 @@ __device__ __forceinline__ float ord_dec(unsigned int u)
 // which all but a bounded number of pills lie); grown until the dense grid
 // fits the table and spans at most 4096 cells per axis.  Non-finite bounds
 // (a diverged state) give an empty grid and raise the non-finite flag.
+//
+// `split`: cells may be cut along x, into four or two where the table has room
+// (inv_x): a pill searches the part of a row of cells that its reach covers
+// (emit_pills), so thinner cells leave out more of it.  Settled strands: 211
+// candidates a pill, 159 with cells cut in four.
 __device__ __forceinline__ Grid make_grid_from(const unsigned int *bounds, int table, bool &ok, float r_cut = -1.f,
-                                               int b_cut = kRadBins - 1)
+                                               int b_cut = kRadBins - 1, bool split = false)
 {
     Grid G;
     float lo[3], hi[3];
@@ -875,7 +880,7 @@ __device__ __forceinline__ Grid make_grid_from(const unsigned int *bounds, int t
             G.lo[c] = 0.f;
             G.dim[c] = 1;
         }
-        G.inv_cell = 0.f;
+        G.inv_cell = G.inv_x = 0.f;
         G.pad = 1;
         return G;
     }
@@ -891,9 +896,18 @@ __device__ __forceinline__ Grid make_grid_from(const unsigned int *bounds, int t
             if (dim[c] < 1) dim[c] = 1;
             tot *= dim[c];
         }
-        G.inv_cell = inv;
+        G.inv_cell = G.inv_x = inv;
         if (tot <= (long long)table) break;
         cell *= 1.26f;
+    }
+    for (int f = 4; split && f > 1; f >>= 1) {
+        const float inv = f * G.inv_cell;
+        const int n = (int)floorf((hi[0] - lo[0]) * inv) + 1;
+        if (n > 0 && (long long)n * dim[1] * dim[2] <= (long long)table) {
+            G.inv_x = inv;
+            dim[0] = n;
+            break;
+        }
     }
     for (int c = 0; c < 3; ++c) {
         G.lo[c] = lo[c];
@@ -916,6 +930,17 @@ __device__ __forceinline__ int cell_coord(float x, float lo, float inv_cell, int
 {
     int i = (int)floorf((x - lo) * inv_cell);
     return min(max(i, 0), dim - 1);
+}
+
+// Cells along an axis that hold every centre within `reach` of x (enlarged by 2^-8
+// for the rounding here and of the centres' own cells).  The reach is taken from
+// the offset into the grid, not from x: far from the origin x - reach would round
+// by more than that.
+__device__ __forceinline__ void cell_range(float x, float reach, float lo, float inv_cell, int dim, int &c0, int &c1)
+{
+    const float d = __fsub_rn(x, lo), r = __fmul_rn(reach, 1.00390625f);
+    c0 = min(max((int)floorf(__fmul_rn(__fsub_rn(d, r), inv_cell)), 0), dim - 1);
+    c1 = min(max((int)floorf(__fmul_rn(__fadd_rn(d, r), inv_cell)), 0), dim - 1);
 }
 
 __device__ __forceinline__ int warp_incl_scan(int v)
@@ -960,7 +985,7 @@ __device__ __forceinline__ float4 bp_sphere(const Params &P, int g)
 
 __device__ __forceinline__ int bp_cell(const Grid &G, float4 sp)
 {
-    const int ix = cell_coord(sp.x, G.lo[0], G.inv_cell, G.dim[0]);
+    const int ix = cell_coord(sp.x, G.lo[0], G.inv_x, G.dim[0]);
     const int iy = cell_coord(sp.y, G.lo[1], G.inv_cell, G.dim[1]);
     const int iz = cell_coord(sp.z, G.lo[2], G.inv_cell, G.dim[2]);
     return ix + G.dim[0] * (iy + G.dim[1] * iz);
@@ -1225,6 +1250,25 @@ __device__ __forceinline__ void flush_rows(const Params &P, const int *buf, int 
     __syncwarp();
 }
 
+// The row's hits of another group than ga, moved up; returns their number.  The
+// groups are looked up for the hits only, four at a time: one candidate in ten is one.
+__device__ __forceinline__ int other_groups(const Params &P, int *row, int cnt, int ga)
+{
+    int n = 0;
+    for (int j = 0; j < cnt; j += 4) {
+        int q[4], g[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            q[t] = j + t < cnt ? row[j + t] : -1;
+            g[t] = q[t] >= 0 ? P.cell_grp[q[t]] : ga;
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            if (g[t] != ga) row[n++] = q[t];
+    }
+    return n;
+}
+
 // spheres_overlap with the components in packed pairs (add and multiply two
 // floats at a time, each rounded as the scalar operation): (b - a) and, in the
 // fourth place, Ra + Rb, then their squares.  na = (-ax, -ay, -az, Ra).
@@ -1244,12 +1288,12 @@ __device__ __forceinline__ bool spheres_overlap2(float4 na, float4 b)
 
 // Candidate pairs of the n pills in the cells, up to the cut, L lanes per pill in cell order
 // (a warp step takes entries p0 .. p0 + 32 / L - 1 of the cell-order copies).
-// Each tests the pills of its own cell after it and those of the 13 forward
-// neighbour cells (dz = 1; dz = 0, dy = 1; dz = dy = 0, dx = 1), so every pair
-// of pills in neighbouring cells is tested once.  Cells are numbered along x,
-// so these are five runs of the cell order: the rest of the own cell with the
-// next one, and four rows of three cells.  A pill's lanes walk its runs end to
-// end, four candidates a lane and step; the warp takes the longest walk's
+// Each tests the pills of its own row after it and those of the four forward
+// rows (dz = 1; dz = 0, dy = 1), within its reach along x (its own radius and the
+// largest), so every pair that overlaps is tested once, from the pill that comes
+// first.  Cells are numbered along x, so these are five runs of the cell order: what
+// follows in the own row, and part of four others.  A pill's lanes walk its runs
+// end to end, four candidates a lane and step; the warp takes the longest walk's
 // number of steps.
 // L = 1 where the pills fill the GPU: settled strands (300,000 pills, 8.8
 // million pairs) take 216 us a search with the oversized pills, against 469 us
@@ -1274,10 +1318,11 @@ __device__ __forceinline__ void emit_pills(const Params &P, const Grid &G, unsig
                 na = make_float4(-sa.x, -sa.y, -sa.z, sa.w);
                 ga = P.cell_grp[p];
                 ia = P.cell_pills[p];
-                const int ix = cell_coord(sa.x, G.lo[0], G.inv_cell, G.dim[0]);
                 const int iy = cell_coord(sa.y, G.lo[1], G.inv_cell, G.dim[1]);
                 const int iz = cell_coord(sa.z, G.lo[2], G.inv_cell, G.dim[2]);
-                const int x0 = max(ix - 1, 0), x1 = min(ix + 1, G.dim[0] - 1) + 1;
+                int x0, x1;
+                cell_range(sa.x, __fadd_rn(fabsf(sa.w), G.r_cut), G.lo[0], G.inv_x, G.dim[0], x0, x1);
+                ++x1;
                 const int r0 = G.dim[0] * (iy + G.dim[1] * iz), ry = G.dim[0], rz = G.dim[0] * G.dim[1];
                 const int *cs = P.cell_start;
                 const bool up = iy + 1 < G.dim[1], down = iy > 0, next = iz + 1 < G.dim[2];
@@ -1301,23 +1346,21 @@ __device__ __forceinline__ void emit_pills(const Params &P, const Grid &G, unsig
             }
             if (!__any_sync(full, q < end)) break;
             float4 cs[4];
-            int cg[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t)
-                if (q + t * L + sub < end) {
-                    cs[t] = P.cell_sph[q + t * L + sub];
-                    cg[t] = P.cell_grp[q + t * L + sub];
-                }
+                if (q + t * L + sub < end) cs[t] = P.cell_sph[q + t * L + sub];
 #pragma unroll
             for (int t = 0; t < 4; ++t)
-                if (q + t * L + sub < end && cg[t] != ga && spheres_overlap2(na, cs[t]) && !(__float_as_uint(cs[t].w) > big))
+                if (q + t * L + sub < end && spheres_overlap2(na, cs[t]) && !(__float_as_uint(cs[t].w) > big))
                     row[cnt++] = q + t * L + sub;
             q += 4 * L;
             if (__any_sync(full, cnt > kLanePairs - 4)) {
+                cnt = other_groups(P, row, cnt, ga);
                 flush_rows(P, buf, cnt, ia, va, lane);
                 cnt = 0;
             }
         }
+        cnt = other_groups(P, row, cnt, ga);
         if (__any_sync(full, cnt > 0)) flush_rows(P, buf, cnt, ia, va, lane);
     }
 }
@@ -1339,7 +1382,7 @@ __device__ __forceinline__ void flush_big(const Params &P, const int *buf, int c
 // the cut, and of the oversized ones those that come after it in the order of
 // descending radius (equal radii by id), so that each pair is found once, from
 // its larger pill, and lies within |Ri| + max(|Ri|, r_cut) of its centre.  The
-// cells of that box (enlarged by 2^-8 for the rounding of its corners) are rows
+// cells of that box (cell_range) are rows
 // of the cell order; 32 rows' ends are loaded at a time.  (Radii can be
 // negative: contacts squeeze them past zero; their bits then sort above every
 // cut.)
@@ -1351,14 +1394,11 @@ __device__ __forceinline__ void emit_big(const Params &P, const Grid &G, unsigne
     const float4 na = make_float4(-si.x, -si.y, -si.z, si.w);
     const float Ri = fabsf(si.w);
     const int grp = P.seg_group[gi], vi = P.pair_v ? P.seg_v0[gi] : 0;
-    const float reach = __fmul_rn(__fadd_rn(Ri, fmaxf(Ri, G.r_cut)), 1.00390625f);
+    const float reach = __fadd_rn(Ri, fmaxf(Ri, G.r_cut));
     const float c[3] = {si.x, si.y, si.z};
     int lo[3], hi[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        lo[k] = cell_coord(__fsub_rn(c[k], reach), G.lo[k], G.inv_cell, G.dim[k]);
-        hi[k] = cell_coord(__fadd_rn(c[k], reach), G.lo[k], G.inv_cell, G.dim[k]);
-    }
+    for (int k = 0; k < 3; ++k) cell_range(c[k], reach, G.lo[k], k ? G.inv_cell : G.inv_x, G.dim[k], lo[k], hi[k]);
     const int ny = hi[1] - lo[1] + 1, rows = ny * (hi[2] - lo[2] + 1);
     int cnt = 0;  // hits in buf (uniform over the warp)
     for (int rb = 0; rb < rows; rb += 32) {

@@ -23,6 +23,7 @@ enum : int { ERR_NONFINITE = 1, ERR_OVERFLOW = 2, ERR_TIMEOUT = 4, ERR_NOCONV = 
 // largest radius.  b_cut: the radius-histogram bin of r_cut (kRadBins - 1: none).
 struct Grid {
     float lo[3];
+    float inv_x;  // cells may be thinner along x (make_grid_from)
     float inv_cell;
     int dim[3];
     int pad;
