@@ -489,28 +489,50 @@ __device__ __forceinline__ void jacobi_vertex(const float4 &qa, const float4 &qb
 // jn = 1/(l_b lv), lv = (l_a + l_b)/2 (Sec. 5 E_bending, Laplacian of Sec. 7.5
 // read as the second derivative, s_bar = 1):
 //  L  C = jn (sn - s) - jp (s - sp),  J = (jp, -(jp + jn), jn)
+// What of it does not depend on the scales: jp, jn, the compliance over h^2 and the
+// approximate inverse of J W J^T + compliance (x fdiv'ed by it is x times that).
+struct LapRest {
+    float jp, jn, at, inv;
+};
+__device__ __forceinline__ LapRest lap_rest(float4 rv2, float wp, float w, float wn, float inv_h2)
+{
+    const float jp = rv2.x, jn = rv2.y, jc = -(jp + jn), at = rv2.z * inv_h2;
+    return {jp, jn, at, fdiv(1.f, wp * jp * jp + w * jc * jc + wn * jn * jn + at)};
+}
+
+__device__ __forceinline__ void laplacian_increments(float sp, float s, float sn, float wp, float w, float wn,
+                                                     const LapRest &T, float &lam, float &dsp, float &ds, float &dsn)
+{
+    const float jc = -(T.jp + T.jn);
+    const float C = T.jn * (sn - s) - T.jp * (s - sp);
+    const float dl = (-C - T.at * lam) * T.inv;
+    lam += dl;
+    dsp = wp * T.jp * dl;
+    ds = w * jc * dl;
+    dsn = wn * T.jn * dl;
+}
+
 __device__ __forceinline__ void laplacian_increments(float sp, float s, float sn, float wp, float w, float wn,
                                                      float4 rv2, float &lam, float inv_h2, float &dsp, float &ds,
                                                      float &dsn)
 {
-    const float jp = rv2.x, jn = rv2.y, jc = -(jp + jn);
-    const float C = jn * (sn - s) - jp * (s - sp);
-    const float at = rv2.z * inv_h2;
-    const float dl = fdiv(-C - at * lam, wp * jp * jp + w * jc * jc + wn * jn * jn + at);
-    lam += dl;
-    dsp = wp * jp * dl;
-    ds = w * jc * dl;
-    dsn = wn * jn * dl;
+    laplacian_increments(sp, s, sn, wp, w, wn, lap_rest(rv2, wp, w, wn, inv_h2), lam, dsp, ds, dsn);
+}
+
+__device__ __forceinline__ void project_laplacian(float &sp, float &s, float &sn, float wp, float w, float wn,
+                                                  const LapRest &T, float &lam)
+{
+    float dsp, ds, dsn;
+    laplacian_increments(sp, s, sn, wp, w, wn, T, lam, dsp, ds, dsn);
+    sp += dsp;
+    s += ds;
+    sn += dsn;
 }
 
 __device__ __forceinline__ void project_laplacian(float &sp, float &s, float &sn, float wp, float w, float wn,
                                                   float4 rv2, float &lam, float inv_h2)
 {
-    float dsp, ds, dsn;
-    laplacian_increments(sp, s, sn, wp, w, wn, rv2, lam, inv_h2, dsp, ds, dsn);
-    sp += dsp;
-    s += ds;
-    sn += dsn;
+    project_laplacian(sp, s, sn, wp, w, wn, lap_rest(rv2, wp, w, wn, inv_h2), lam);
 }
 
 // ---------------------------------------------------------------- pills
