@@ -455,45 +455,47 @@ __device__ __forceinline__ void zero_lam(SlotLam &L)
 __device__ __forceinline__ void sweep(SmemRod sX, SmemRod sQ, const SlotRest &R, SlotLam &L, float inv_h2,
                                       bool vol, const float4 *__restrict__ RV2 = nullptr)
 {
-    const int lv = R.lv, ls = R.ls;
+    const int lv = R.lv;
+    // the slot's elements: of one parity they lie side by side (SmemRod)
+    float4 *const x0 = &sX[lv], *const x1 = &sX[lv + 1], *const q0 = &sQ[R.ls], *const q1 = &sQ[R.ls + 1];
     // colour 0: even segments
     if (R.has0) {
-        float4 xa = sX[lv], xb = sX[lv + 1], q = sQ[ls];
+        float4 xa = x0[0], xb = x1[0], q = q0[0];
         project_segment(xa, xb, q, R.w0, R.w1, R.ws0, R.ws1, R.rs00, R.rs10, L.s0, L.x0, inv_h2, vol);
-        sX[lv] = xa;
-        sX[lv + 1] = xb;
-        sQ[ls] = q;
+        x0[0] = xa;
+        x1[0] = xb;
+        q0[0] = q;
     }
     __syncthreads();
     // colour 1: odd segments
     if (R.has1) {
-        float4 xa = sX[lv + 1], xb = sX[lv + 2], q = sQ[ls + 1];
+        float4 xa = x1[0], xb = x0[1], q = q1[0];
         project_segment(xa, xb, q, R.w1, R.w2, R.ws1, R.ws2, R.rs01, R.rs11, L.s1, L.x1, inv_h2, vol);
-        sX[lv + 1] = xa;
-        sX[lv + 2] = xb;
-        sQ[ls + 1] = q;
+        x1[0] = xa;
+        x0[1] = xb;
+        q1[0] = q;
     }
     __syncthreads();
     // colour 2: even interior vertices (2p+2), segments 2p+1 and 2p+2
     if (R.hasv2) {
-        float4 qa = sQ[ls + 1], qb = sQ[ls + 2];
-        float s = sX[lv + 2].w;
-        project_vertex(qa, qb, s, sX[lv + 1].w, sX[lv + 3].w, R.rs01.x, R.l2, R.rs01.y, R.im2, R.ws2, R.rv02, R.aB2,
-                       R.aV2, L.b2, L.v2, inv_h2, vol);
-        sQ[ls + 1] = qa;
-        sQ[ls + 2] = qb;
-        sX[lv + 2].w = s;
+        float4 qa = q1[0], qb = q0[1];
+        float s = x0[1].w;
+        project_vertex(qa, qb, s, x1[0].w, x1[1].w, R.rs01.x, R.l2, R.rs01.y, R.im2, R.ws2, R.rv02, R.aB2, R.aV2,
+                       L.b2, L.v2, inv_h2, vol);
+        q1[0] = qa;
+        q0[1] = qb;
+        x0[1].w = s;
     }
     __syncthreads();
     // colour 3: odd interior vertices (2p+1), segments 2p and 2p+1
     if (R.has1) {
-        float4 qa = sQ[ls], qb = sQ[ls + 1];
-        float s = sX[lv + 1].w;
-        project_vertex(qa, qb, s, sX[lv].w, sX[lv + 2].w, R.rs00.x, R.rs01.x, R.rs00.y, R.rs01.y, R.ws1, R.rv01,
-                       R.aB1, R.aV1, L.b1, L.v1, inv_h2, vol);
-        sQ[ls] = qa;
-        sQ[ls + 1] = qb;
-        sX[lv + 1].w = s;
+        float4 qa = q0[0], qb = q1[0];
+        float s = x1[0].w;
+        project_vertex(qa, qb, s, x0[0].w, x0[1].w, R.rs00.x, R.rs01.x, R.rs00.y, R.rs01.y, R.ws1, R.rv01, R.aB1,
+                       R.aV1, L.b1, L.v1, inv_h2, vol);
+        q0[0] = qa;
+        q1[0] = qb;
+        x1[0].w = s;
     }
     __syncthreads();
     if (RV2) {
