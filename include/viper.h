@@ -364,12 +364,12 @@ int viper_contact_stats(viper_scene *scene, long long out[3]);
  *
  * Every kernel of the frame covers all scenes of the call: its grid is the
  * concatenation of the scenes' grids, so a frame of S substeps and I >= 1
- * iterations costs S (2 I + 2) + 3 launches (contacts, skinning) however
+ * iterations costs S (2 I + 3) + 3 launches (contacts, skinning) however
  * many scenes it carries.
  * Scenes with contacts or half-planes whose rods all fit the shared-memory
  * kernel (every scene whose rods are at most resident_max long) run the
- * contact-path sequence; such scenes without contacts run one launch per
- * substep; the rest are stepped one by one as viper_step would.  Each scene
+ * contact-path sequence; such scenes without contacts run one launch for
+ * all substeps; the rest are stepped one by one as viper_step would.  Each scene
  * computes what viper_step computes for it (to FP32 rounding: the same
  * device code), and its result does not depend on the other scenes of the
  * call.

@@ -870,9 +870,7 @@ __global__ void __launch_bounds__(kElemThreads) batch_skin_kernel(BatchArgs A)
 // ---------------------------------------------------------------- host side
 namespace {
 
-// Launch with programmatic stream serialisation (the kernel's prologue may
-// overlap its predecessor; see batch_enter).
-// launch_clusters: in thread-block clusters of `ctas`.
+// launch_dependent in thread-block clusters of `ctas`.
 template <typename... KArgs, typename... Args>
 void launch_clusters(void (*kernel)(KArgs...), int grid, int ctas, int block, int smem, cudaStream_t st, Args... args)
 {
@@ -888,14 +886,8 @@ void launch_clusters(void (*kernel)(KArgs...), int grid, int ctas, int block, in
     at[1].val.clusterDim.x = ctas;
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = ctas > 1 ? 2 : 1;
+    cfg.numAttrs = 2;
     cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
-template <typename... KArgs, typename... Args>
-void launch(void (*kernel)(KArgs...), int grid, int block, int smem, cudaStream_t st, Args... args)
-{
-    launch_clusters(kernel, grid, 1, block, smem, st, args...);
 }
 
 // CTAs of the cluster that builds a scene's grid: eight where that fills no more
@@ -1090,22 +1082,22 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
                                 sh.slice_cap, sh.groups_cap);
             });
         } else {
-            go(PROF_BROADPHASE, [&] { launch(batch_bounds_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
-            go(PROF_BROADPHASE, [&] { launch(batch_count_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
-            go(PROF_BROADPHASE, [&] { launch(batch_scan_kernel, tot[K_SCAN], kScanThreadsB, 0, bs, A); });
-            go(PROF_BROADPHASE, [&] { launch(batch_scatter_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
+            go(PROF_BROADPHASE, [&] { launch_dependent(batch_bounds_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
+            go(PROF_BROADPHASE, [&] { launch_dependent(batch_count_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
+            go(PROF_BROADPHASE, [&] { launch_dependent(batch_scan_kernel, tot[K_SCAN], kScanThreadsB, 0, bs, A); });
+            go(PROF_BROADPHASE, [&] { launch_dependent(batch_scatter_kernel, tot[K_PILL], kElemThreads, 0, bs, A); });
         }
         go(PROF_PAIRS, [&] {
-            launch(sh.small ? batch_emit_kernel<kEmitLanesSmall> : batch_emit_kernel<1>, tot[K_EMIT], 32 * kEmitWarpsB, 0, bs, A);
+            launch_dependent(sh.small ? batch_emit_kernel<kEmitLanesSmall> : batch_emit_kernel<1>, tot[K_EMIT], 32 * kEmitWarpsB, 0, bs, A);
         });
     };
     // the broadphase on a second branch beside the first sweep (not while profiling:
     // the per-class events bracket one stream)
     const bool forked = fork && fork->side && tot[K_PILL] > 0 && (!prof || prof->prof_class == PROF_NONE);
     auto contact = [&](int first) {
-        go(PROF_CONTACT, [&] { launch(batch_contact_kernel, tot[K_CONTACT], kElemThreads, 0, st, A, first); });
+        go(PROF_CONTACT, [&] { launch_dependent(batch_contact_kernel, tot[K_CONTACT], kElemThreads, 0, st, A, first); });
     };
-    if (tot[K_WARM] > 0) go(PROF_ELEM, [&] { launch(batch_warm_kernel, tot[K_WARM], kElemThreads, 0, st, A); });
+    if (tot[K_WARM] > 0) go(PROF_ELEM, [&] { launch_dependent(batch_warm_kernel, tot[K_WARM], kElemThreads, 0, st, A); });
     if (cp && iterations > 0) {
         // per substep: [finish + predict + sweep 0] | grid | emit | contact | {sweep | contact} x (I - 1)
         for (int k = 0; k < substeps; ++k) {
@@ -1114,41 +1106,41 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
                 // advance | [grid, pair search] beside [first sweep] | contact ...; the grid and
                 // the pair search take longer than the sweep, so they follow on the main
                 // stream, where their prologues overlap what is before them
-                go(PROF_ELEM, [&] { launch(batch_advance_kernel, tot[K_ELEM], kElemThreads, 0, st, A, k > 0 ? 1 : 0, tau); });
+                go(PROF_ELEM, [&] { launch_dependent(batch_advance_kernel, tot[K_ELEM], kElemThreads, 0, st, A, k > 0 ? 1 : 0, tau); });
                 if (cudaEventRecord(fork->ev_fork, st) != cudaSuccess ||
                     cudaStreamWaitEvent(fork->side, fork->ev_fork, 0) != cudaSuccess)
                     return -1;
                 broadphase(st);
-                go(PROF_ROD, [&] { launch(batch_rod_kernel, tot[K_ROD], threads, smem, fork->side, A, 1, 0); });
+                go(PROF_ROD, [&] { launch_dependent(batch_rod_kernel, tot[K_ROD], threads, smem, fork->side, A, 1, 0); });
                 if (cudaEventRecord(fork->ev_join, fork->side) != cudaSuccess ||
                     cudaStreamWaitEvent(st, fork->ev_join, 0) != cudaSuccess)
                     return -1;
             } else {
-                go(PROF_ROD, [&] { launch(batch_rod_first_kernel, tot[K_ROD], threads, smem, st, A, k > 0 ? 1 : 0, tau); });
+                go(PROF_ROD, [&] { launch_dependent(batch_rod_first_kernel, tot[K_ROD], threads, smem, st, A, k > 0 ? 1 : 0, tau); });
                 broadphase(st);
             }
             contact(1);
             for (int i = 1; i < iterations; ++i) {
-                go(PROF_ROD, [&] { launch(batch_rod_kernel, tot[K_ROD], threads, smem, st, A, 0, 1); });
+                go(PROF_ROD, [&] { launch_dependent(batch_rod_kernel, tot[K_ROD], threads, smem, st, A, 0, 1); });
                 contact(0);
             }
             if (tot[K_BUNDLE] > 0)
-                go(PROF_ELEM, [&] { launch(batch_bundle_kernel, tot[K_BUNDLE], kElemThreads, 0, st, A); });
+                go(PROF_ELEM, [&] { launch_dependent(batch_bundle_kernel, tot[K_BUNDLE], kElemThreads, 0, st, A); });
         }
-        go(PROF_ELEM, [&] { launch(batch_finish_kernel, tot[K_ELEM], kElemThreads, 0, st, A, 1); });
+        go(PROF_ELEM, [&] { launch_dependent(batch_finish_kernel, tot[K_ELEM], kElemThreads, 0, st, A, 1); });
     } else if (!cp) {
-        go(PROF_ROD, [&] { launch(batch_rod_frame_kernel, tot[K_ROD], threads, smem, st, A, substeps, iterations); });
+        go(PROF_ROD, [&] { launch_dependent(batch_rod_frame_kernel, tot[K_ROD], threads, smem, st, A, substeps, iterations); });
     } else {
         // contact path without iterations: prediction, broadphase, velocity update
         for (int k = 0; k < substeps; ++k) {
             const float tau = (float)((double)(k + 1) / substeps);  // as the one-scene path
-            go(PROF_ELEM, [&] { launch(batch_predict_kernel, tot[K_ELEM], kElemThreads, 0, st, A, tau); });
+            go(PROF_ELEM, [&] { launch_dependent(batch_predict_kernel, tot[K_ELEM], kElemThreads, 0, st, A, tau); });
             broadphase(st);
-            go(PROF_ELEM, [&] { launch(batch_finish_kernel, tot[K_ELEM], kElemThreads, 0, st, A, 0); });
+            go(PROF_ELEM, [&] { launch_dependent(batch_finish_kernel, tot[K_ELEM], kElemThreads, 0, st, A, 0); });
         }
     }
-    go(PROF_ELEM, [&] { launch(batch_end_kernel, tot[K_END], kElemThreads, 0, st, A); });
-    if (tot[K_MESH] > 0) go(PROF_LBS, [&] { launch(batch_skin_kernel, tot[K_MESH], kElemThreads, 0, st, A); });
+    go(PROF_ELEM, [&] { launch_dependent(batch_end_kernel, tot[K_END], kElemThreads, 0, st, A); });
+    if (tot[K_MESH] > 0) go(PROF_LBS, [&] { launch_dependent(batch_skin_kernel, tot[K_MESH], kElemThreads, 0, st, A); });
     return cudaGetLastError() == cudaSuccess ? L : -1;
 }
 

@@ -587,26 +587,27 @@ void enqueue_frame(viper_scene *s, float dt, int substeps, int iterations)
                 launch_advance(s, k > 0, pills);
             else
                 launch_predict(s, 0, nv, 0, ns, true);
-            // the broadphase only needs the predicted state: run it on a second
-            // branch beside the first constraint sweep, join before the first contact pass
-            bool forked = false;
-            if (pills && iterations > 0) {
+            // the broadphase only needs the predicted state: the first constraint sweep
+            // runs beside it on a second branch, joined before the first contact pass (the
+            // broadphase, the longer of the two, on the main branch, where every kernel
+            // overlaps the end of the one before)
+            const bool forked = pills && iterations > 0;
+            if (forked) {
                 cudaEventRecord(s->ev_fork, s->stream);
                 cudaStreamWaitEvent(s->side, s->ev_fork, 0);
-                s->ls = s->side;
-                launch_broadphase(s);
-                cudaEventRecord(s->ev_join, s->side);
-                s->ls = s->stream;
-                forked = true;
-            } else if (pills) {
-                launch_broadphase(s);
             }
+            if (pills) launch_broadphase(s, fused);
             for (int it = 0; it < iterations; ++it) {
+                if (it == 0 && forked) s->ls = s->side;
                 launch_rod_iter(s, it == 0, it > 0);
-                if (it == 0 && forked) cudaStreamWaitEvent(s->stream, s->ev_join, 0);
                 if (s->resident_nv < nv) {
                     if (it > 0) launch_apply(s, s->resident_nv, nv);
                     for (int c = 0; c < n_colours(s); ++c) launch_colour(s, c, s->col_list[c], s->col_n[c]);
+                }
+                if (it == 0 && forked) {
+                    cudaEventRecord(s->ev_join, s->side);
+                    s->ls = s->stream;
+                    cudaStreamWaitEvent(s->stream, s->ev_join, 0);
                 }
                 launch_contacts(s);
             }

@@ -35,6 +35,8 @@ __global__ void __launch_bounds__(kBpThreads) bp_bounds_kernel(Params P)
     for (int b = threadIdx.x; b < kRadBins; b += blockDim.x) hist[b] = 0;
     if (threadIdx.x < 8) s_bounds[threadIdx.x] = 0u;
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY}, mr = 0.f;
     const int lane = threadIdx.x & 31;
     for (int g0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); g0 < P.ns; g0 += gridDim.x * blockDim.x) {
@@ -62,6 +64,8 @@ __global__ void __launch_bounds__(kBpThreads) bp_bounds_kernel(Params P)
 __global__ void __launch_bounds__(kBpThreads) bp_count_kernel(Params P)
 {
     __shared__ int sh[kRadBins + 33];
+    pdl_wait();
+    pdl_trigger();
     float r_cut;
     const int b_cut = choose_cut<kRadBins / kBpThreads>(P.bp_hist, P.big_cap, 1, ord_dec(P.bounds[6]), sh, &r_cut);
     bool ok;
@@ -87,6 +91,8 @@ __global__ void __launch_bounds__(kBpThreads) bp_count_kernel(Params P)
 // cell_count is returned to zero here (each pill takes one slot), ready for the next substep
 __global__ void bp_scatter_kernel(Params P)
 {
+    pdl_wait();
+    pdl_trigger();
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.ns; g += gridDim.x * blockDim.x) {
         const int cell = P.cell_of[g];
         scatter_pill(P, g, cell, P.cell_start[cell]);
@@ -99,6 +105,8 @@ constexpr int kEmitWarps = 8;
 __global__ void __launch_bounds__(32 * kEmitWarps, 4) bp_emit_kernel(Params P)
 {
     __shared__ int buf[kEmitWarps][kEmitBuf];
+    pdl_wait();
+    pdl_trigger();
     const Grid G = *P.grid;
     if (G.pad) return;  // no valid grid: no candidates
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -120,6 +128,8 @@ constexpr int kScanThreads = 1024, kScanPer = 4, kScanTile = kScanThreads * kSca
 __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(const int *in, int n, int *tile_sums, const Grid *g)
 {
     __shared__ int ws[33];
+    pdl_wait();
+    pdl_trigger();
     n = grid_cells(g, n);
     int base = blockIdx.x * kScanTile + threadIdx.x * kScanPer;
     int s = 0;
@@ -135,6 +145,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_sums_kernel(int *tile_sums,
                                                                  const Grid *g)
 {
     __shared__ int ws[33];
+    pdl_wait();
+    pdl_trigger();
     int base = threadIdx.x * kScanPer;
     int v[kScanPer], s = 0;
 #pragma unroll
@@ -156,6 +168,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(const int *in,
                                                                   const Grid *g)
 {
     __shared__ int ws[33];
+    pdl_wait();
+    pdl_trigger();
     n = grid_cells(g, n);
     if (blockIdx.x * kScanTile >= n) return;  // uniform over the CTA
     int base = blockIdx.x * kScanTile + threadIdx.x * kScanPer;
@@ -178,6 +192,8 @@ constexpr int kSmallPer = 16;
 __global__ void __launch_bounds__(kScanThreads) scan_small_kernel(const int *in, int n, int *out, const Grid *g)
 {
     __shared__ int ws[33];
+    pdl_wait();
+    pdl_trigger();
     n = grid_cells(g, n);
     const int base = threadIdx.x * kSmallPer;
     int v[kSmallPer], s = 0;
@@ -200,7 +216,7 @@ static void scan(viper_scene *s, cudaStream_t st, int *tmp, const int *in, int n
 {
     if (n <= kScanThreads * kSmallPer) {
         ProfScope ps(s, PROF_BROADPHASE);
-        scan_small_kernel<<<1, kScanThreads, 0, st>>>(in, n, out, g);
+        launch_dependent(scan_small_kernel, 1, kScanThreads, 0, st, in, n, out, g);
         if (s) s->launches += 1;
         return;
     }
@@ -208,48 +224,51 @@ static void scan(viper_scene *s, cudaStream_t st, int *tmp, const int *in, int n
     if (tiles < 1) tiles = 1;
     {
         ProfScope ps(s, PROF_BROADPHASE);
-        scan_tiles_kernel<<<tiles, kScanThreads, 0, st>>>(in, n, tmp, g);
+        launch_dependent(scan_tiles_kernel, tiles, kScanThreads, 0, st, in, n, tmp, g);
     }
     {
         ProfScope ps(s, PROF_BROADPHASE);
-        scan_sums_kernel<<<1, kScanThreads, 0, st>>>(tmp, tiles, out, n, g);
+        launch_dependent(scan_sums_kernel, 1, kScanThreads, 0, st, tmp, tiles, out, n, g);
     }
     {
         ProfScope ps(s, PROF_BROADPHASE);
-        scan_apply_kernel<<<tiles, kScanThreads, 0, st>>>(in, n, tmp, out, g);
+        launch_dependent(scan_apply_kernel, tiles, kScanThreads, 0, st, in, n, tmp, out, g);
     }
     if (s) s->launches += 3;
 }
 
 
-void broadphase_enqueue(const Params &P, cudaStream_t st, int *scan_tmp, viper_scene *s)
+void broadphase_enqueue(const Params &P, cudaStream_t st, int *scan_tmp, viper_scene *s, bool cleared)
 {
     const int grid = (P.ns + 255) / 256 < 4 * device_sm_count() ? (P.ns + 255) / 256 + 1 : 4 * device_sm_count();
-    cudaMemsetAsync(P.bounds, 0, kBoundsWords * sizeof(unsigned int), st);
+    if (!cleared) cudaMemsetAsync(P.bounds, 0, kBoundsWords * sizeof(unsigned int), st);
     {
         ProfScope ps(s, PROF_BROADPHASE);
-        bp_bounds_kernel<<<grid, kBpThreads, 0, st>>>(P);
+        launch_dependent(bp_bounds_kernel, grid, kBpThreads, 0, st, P);
     }
     {
         ProfScope ps(s, PROF_BROADPHASE);
-        bp_count_kernel<<<grid, kBpThreads, 0, st>>>(P);
+        launch_dependent(bp_count_kernel, grid, kBpThreads, 0, st, P);
     }
     scan(s, st, scan_tmp, P.cell_count, P.table, P.cell_start, P.grid);
     {
         ProfScope ps(s, PROF_BROADPHASE);
-        bp_scatter_kernel<<<grid, 256, 0, st>>>(P);
+        launch_dependent(bp_scatter_kernel, grid, 256, 0, st, P);
     }
     {
         int eg = (P.ns + 32 * kEmitWarps - 1) / (32 * kEmitWarps);  // a thread per pill
         if (eg > 8 * device_sm_count()) eg = 8 * device_sm_count();
         if (eg < 1) eg = 1;
         ProfScope ps(s, PROF_PAIRS);
-        bp_emit_kernel<<<eg, 32 * kEmitWarps, 0, st>>>(P);
+        launch_dependent(bp_emit_kernel, eg, 32 * kEmitWarps, 0, st, P);
     }
     if (s) s->launches += 4;
 }
 
-void launch_broadphase(viper_scene *s) { broadphase_enqueue(s->P, s->ls, s->d_scan_tmp, s); }
+void launch_broadphase(viper_scene *s, bool cleared)
+{
+    broadphase_enqueue(s->P, s->ls, s->d_scan_tmp, s, cleared);
+}
 
 // ---------------------------------------------------------------- contact pass
 constexpr int kContactThreads = 256;
@@ -259,6 +278,7 @@ __global__ void __launch_bounds__(kContactThreads, 4) contact_kernel(Params P)
     __shared__ unsigned long long stats[2];
     if (threadIdx.x < 2) stats[threadIdx.x] = 0;
     __syncthreads();
+    pdl_wait();
     const int np_all = *P.npairs;
     const int np = min(np_all, P.max_pairs);
     if (blockIdx.x == 0 && threadIdx.x == 0 && np_all > P.max_pairs) atomicOr(P.err, ERR_OVERFLOW);
@@ -283,6 +303,9 @@ __global__ void __launch_bounds__(kContactThreads, 4) contact_kernel(Params P)
         atomicAdd(stats, (unsigned long long)counts.x);
         atomicAdd(stats + 1, (unsigned long long)counts.y);
     }
+    // not before the pairs: sweeps waiting beside the pass slow it (3,000 settled strands, a
+    // frame 2.52 ms against 2.41)
+    pdl_trigger();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nvp; i += threads) contact_planes(P, i, at);
     if (P.contact_stats) {
         __syncthreads();
@@ -314,7 +337,7 @@ void launch_contacts(viper_scene *s)
     const int cap = s->P.max_pairs + (s->P.n_planes > 0 ? s->P.nv : 0);
     const int grid = contact_grid(cap);
     ProfScope ps(s, PROF_CONTACT);
-    contact_kernel<<<grid, kContactThreads, 0, s->ls>>>(contact_path_params(s));
+    launch_dependent(contact_kernel, grid, kContactThreads, 0, s->ls, contact_path_params(s));
     s->launches++;
 }
 

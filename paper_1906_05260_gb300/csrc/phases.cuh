@@ -50,6 +50,25 @@ inline int raise_smem_limit(const void *fn, int bytes)
 // predecessor grid has completed and its memory is visible (a no-op for a
 // normal launch); pdl_trigger lets the successor be scheduled once every CTA
 // of this grid has issued it.
+//
+// launch_dependent launches so.  Every kernel that it launches calls pdl_wait before it
+// touches anything another kernel writes (and before it ends, so that a kernel's
+// end implies its predecessors').
+template <typename... KArgs, typename... Args>
+inline void launch_dependent(void (*kernel)(KArgs...), int grid, int block, int smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -36,6 +36,10 @@ __global__ void predict_kernel(Params P, int v0, int v1, int s0, int s1, int con
 __global__ void advance_kernel(Params P, int finish_prev, int world)
 {
     const bool fin = finish_prev != 0;
+    pdl_wait();
+    pdl_trigger();
+    if (world)  // ready for this substep's broadphase
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kBoundsWords; i += gridDim.x * blockDim.x) P.bounds[i] = 0u;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.nv + P.ns; i += gridDim.x * blockDim.x) {
         if (i < P.nv) {
             AdvanceVertex V;
@@ -51,6 +55,8 @@ __global__ void advance_kernel(Params P, int finish_prev, int world)
 
 __global__ void finish_kernel(Params P, int v0, int v1, int s0, int s1, int apply)
 {
+    pdl_wait();
+    pdl_trigger();
     const int nvr = v1 - v0, total = nvr + (s1 - s0);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         if (i < nvr)
@@ -209,7 +215,10 @@ __global__ void __maxnreg__(96) rod_kernel(Params P, int first, int apply)
     extern __shared__ float4 smem[];
     RodStage S;
     rod_stage_rest(P, blockIdx.x, first != 0, S);
-    rod_stage_state(P, S, smem);
+    if (!first) rod_stage_state(P, S, smem);  // after a contact pass: it changes no state
+    pdl_wait();
+    pdl_trigger();
+    if (first) rod_stage_state(P, S, smem);
     rod_run(P, S, apply != 0, smem);
 }
 
@@ -239,7 +248,7 @@ void launch_advance(viper_scene *s, bool finish_prev, bool world)
 {
     const int n = s->nv + s->ns;
     ProfScope ps(s, PROF_ELEM);
-    advance_kernel<<<grid_for(n, 256), 256, 0, s->ls>>>(s->P, finish_prev ? 1 : 0, world ? 1 : 0);
+    launch_dependent(advance_kernel, grid_for(n, 256), 256, 0, s->ls, s->P, finish_prev ? 1 : 0, world ? 1 : 0);
     s->launches++;
 }
 
@@ -248,7 +257,7 @@ void launch_finish(viper_scene *s, int v0, int v1, int s0, int s1, bool apply)
     int n = (v1 - v0) + (s1 - s0);
     if (n <= 0) return;
     ProfScope ps(s, PROF_ELEM);
-    finish_kernel<<<grid_for(n, 256), 256, 0, s->ls>>>(s->P, v0, v1, s0, s1, apply ? 1 : 0);
+    launch_dependent(finish_kernel, grid_for(n, 256), 256, 0, s->ls, s->P, v0, v1, s0, s1, apply ? 1 : 0);
     s->launches++;
 }
 
@@ -318,8 +327,8 @@ void launch_rod_iter(viper_scene *s, bool first, bool apply)
 {
     if (s->n_items <= 0) return;
     ProfScope ps(s, PROF_ROD);
-    rod_kernel<<<s->n_items, s->block_threads, s->smem_iter, s->ls>>>(contact_path_params(s), first ? 1 : 0,
-                                                                      apply ? 1 : 0);
+    launch_dependent(rod_kernel, s->n_items, s->block_threads, s->smem_iter, s->ls, contact_path_params(s), first ? 1 : 0,
+                     apply ? 1 : 0);
     s->launches++;
 }
 

@@ -263,10 +263,11 @@ void launch_colour(viper_scene *s, int colour, const int *list, int n);
 void launch_rod_frame(viper_scene *s, int substeps, int n_iter);
 void launch_rod_iter(viper_scene *s, bool first, bool apply);
 void launch_apply(viper_scene *s, int v_begin, int v_end);
-void launch_broadphase(viper_scene *s);
+void launch_broadphase(viper_scene *s, bool cleared = false);
 // Enqueue the broadphase on `st` for the pills described by P (Xpred, bp_rbar,
 // seg_v0, seg_group, grid buffers, pairs, npairs); `s` may be null (no scene).
-void broadphase_enqueue(const Params &P, cudaStream_t st, int *scan_tmp, viper_scene *s);
+// `cleared`: the kBoundsWords words have been zeroed on st (advance_kernel does).
+void broadphase_enqueue(const Params &P, cudaStream_t st, int *scan_tmp, viper_scene *s, bool cleared = false);
 void launch_contacts(viper_scene *s);
 // Params of the multi-kernel contact path's sweeps and contact passes: the
 // scene's, with the world pack when every rod runs in the shared-memory sweep.
