@@ -392,10 +392,10 @@ def bench_batching(V, torch, flush, dist, peaks, peak_kind, fp32_peak_tflops, fr
                 tot += ms_k
                 nl += n
             us = 1e3 * tot / max(nl, 1)
-            per_launch = sc.substeps if mode == V.SOLVER_FRAME else 1  # substeps per launch
+            per_launch = sc.substeps  # either solver: all substeps in one launch (no contacts)
             flops = sc.nv * sc.iterations * ROD_FLOP_PER_VERTEX_SWEEP * per_launch
-            bytes_ = sc.nv * 140.0 * (1 if mode == V.SOLVER_FRAME else 1)  # state in/out + rest once per launch
-            out["rod_kernel" if mode == V.SOLVER_BATCHED else "frame_kernel"] = {
+            bytes_ = sc.nv * 140.0  # state in/out + rest once per launch
+            out["rod_frame_kernel" if mode == V.SOLVER_BATCHED else "frame_kernel"] = {
                 "us_per_launch": us, "launches_per_frame": nl / min(frames, 10),
                 "alu": {"achieved": flops / (us * 1e-6) / 1e12, "peak": fp32_peak_tflops, "unit": "TFLOP/s",
                         "frac": flops / (us * 1e-6) / 1e12 / fp32_peak_tflops},
