@@ -1031,18 +1031,20 @@ __device__ __forceinline__ int bp_cell(const Grid &G, float4 sp)
     return ix + G.dim[0] * (iy + G.dim[1] * iz);
 }
 
-// Bounding sphere of pill g into P.spheres, folded into this thread's running bounds.
+// Bounding sphere of pill g into P.spheres, folded into this thread's running bounds
+// (the radius by its size: contacts squeeze radii past zero, and spheres_overlap squares
+// the sum, so the search's reach is that of the largest size).
 __device__ __forceinline__ void bound_pill(const Params &P, int g, float mn[3], float mx[3], float &mr)
 {
     const float4 sp = bp_sphere(P, g);
     P.spheres[g] = sp;
     mn[0] = fminf(mn[0], sp.x); mn[1] = fminf(mn[1], sp.y); mn[2] = fminf(mn[2], sp.z);
     mx[0] = fmaxf(mx[0], sp.x); mx[1] = fmaxf(mx[1], sp.y); mx[2] = fmaxf(mx[2], sp.z);
-    mr = fmaxf(mr, sp.w);
+    mr = fmaxf(mr, fabsf(sp.w));
 }
 
 // Warp-wide min/max of the running bounds, merged into `bounds` by lane 0:
-// bounds[0..2] = enc(-min c), bounds[3..5] = enc(max c), bounds[6] = enc(max R),
+// bounds[0..2] = enc(-min c), bounds[3..5] = enc(max c), bounds[6] = enc(max |R|),
 // all zero before the first merge.  Every lane of the warp must call it.
 __device__ __forceinline__ void merge_bounds_to(unsigned int *bounds, float mn[3], float mx[3], float mr)
 {
