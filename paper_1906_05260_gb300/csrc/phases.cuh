@@ -51,9 +51,18 @@ inline int raise_smem_limit(const void *fn, int bytes)
 // normal launch); pdl_trigger lets the successor be scheduled once every CTA
 // of this grid has issued it.
 //
-// launch_dependent launches so.  Every kernel that it launches calls pdl_wait before it
-// touches anything another kernel writes (and before it ends, so that a kernel's
-// end implies its predecessors').
+// launch_dependent launches so.  The rule for every kernel that it launches:
+//  * pdl_wait comes before pdl_trigger and before the end, on every way through the
+//    kernel.  A CTA that may run therefore knows that whatever ran before its
+//    predecessor has completed: the predecessor's CTAs have all passed their own wait.
+//  * Ahead of its pdl_wait a kernel writes nothing outside its CTA, and reads only what its
+//    predecessor does not write: tables of the call, and what was written two launches
+//    back or earlier (the sweeps after a contact pass read X, Q and the multipliers so,
+//    the advance kernel Xp, Qp and, without bundles, X and Q, the later contact passes
+//    and the sweeps the pair count).  A pdl_trigger moved ahead of a pdl_wait, or
+//    another kernel put between, would make a race of that.
+//  * What the predecessor writes is read by coherent loads after the wait: no .nc form
+//    and no __ldg, which ask for memory that nothing writes while the kernel is resident.
 template <typename... KArgs, typename... Args>
 inline void launch_dependent(void (*kernel)(KArgs...), int grid, int block, int smem, cudaStream_t st, Args... args)
 {
@@ -71,6 +80,18 @@ inline void launch_dependent(void (*kernel)(KArgs...), int grid, int block, int 
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Two float4 on a 32-byte boundary in one 256-bit load (sm_100 and later): one request
+// per lane for a gather of 32-byte records, instead of two.  Coherent, and not moved
+// across a pdl_wait: the records (pill packs, skinning frames) are written by the
+// kernel before, which a programmatic launch overlaps.
+__device__ __forceinline__ void ld_record(const float4 *p, float4 &a, float4 &b)
+{
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+                 : "l"(p)
+                 : "memory");
+}
 
 // ================================================================ rods
 // Pin target in the rod's local frame.  Bone pose at substep fraction tau:
@@ -1640,18 +1661,11 @@ __device__ __forceinline__ bool contact_may_touch(const PillPair &Q)
 // rounding; a NaN or infinite n certifies nothing).  One 256-bit load per
 // pill and about 65 operations; from the four vertices, with IEEE divisions and
 // square roots, the test took 350 instructions a warp.
-__device__ __forceinline__ void ld_pill_box(const float4 *b, float4 &m, float4 &d)
-{
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(m.x), "=f"(m.y), "=f"(m.z), "=f"(m.w), "=f"(d.x), "=f"(d.y), "=f"(d.z), "=f"(d.w)
-        : "l"(b));
-}
-
 __device__ __forceinline__ bool boxes_may_touch(const Params &P, int2 pv)
 {
     float4 am, ad, bm, bd;
-    ld_pill_box(P.PB + 2 * (size_t)pv.x, am, ad);
-    ld_pill_box(P.PB + 2 * (size_t)pv.y, bm, bd);
+    ld_record(P.PB + 2 * (size_t)pv.x, am, ad);
+    ld_record(P.PB + 2 * (size_t)pv.y, bm, bd);
     const V3 e = xyz(am) - xyz(bm), da = xyz(ad), db = xyz(bd);
     const float lim = am.w + bm.w;
     const float ee = dot(e, e), ea = dot(e, da), eb = dot(e, db);
@@ -1912,17 +1926,6 @@ __device__ __forceinline__ void lbs_frame_at(const Params &P, const float4 *__re
     f[1] = make_float4(t.x, t.y, t.z, sm);
 }
 
-// One 32-byte frame in a single 256-bit read-only load (sm_100 and later): the
-// frame array starts 256-byte aligned and a frame is 32 bytes, so each frame is
-// one aligned sector and a warp's random gather costs one L1 request per lane
-// instead of two.
-__device__ __forceinline__ void ld_frame(const float4 *f, float4 &r, float4 &ts)
-{
-    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w), "=f"(ts.x), "=f"(ts.y), "=f"(ts.z), "=f"(ts.w)
-                 : "l"(f));
-}
-
 // Skinned position of mesh vertex i: sum_k w_k T_k Tbar_k^-1 rest_i over its
 // four frames, from the vertex's rest position, frame ids and weights.  A
 // frame is 32 bytes: the relative rotation r = R_j Rbar_j^T as a unit
@@ -1946,7 +1949,7 @@ __device__ __forceinline__ float4 lbs_blend(float4 p, int4 id, float4 ww, int ns
             r = frames[ids[k]];
             ts = frames[ns + ids[k]];
         } else {
-            ld_frame(frames + kLbsFrame * (size_t)ids[k], r, ts);
+            ld_record(frames + kLbsFrame * (size_t)ids[k], r, ts);
         }
         const V3 y = qrot(r, v3(p.x, p.y, p.z));
         ox += wv[k] * (ts.w * y.x + ts.x);
