@@ -19,10 +19,15 @@ namespace {
 constexpr double kPi = 3.14159265358979323846;
 Alloc g_alloc;  // process-wide default for new scenes
 
+// The error is the calling function's result; it is not left behind for the next call
+// to find as its own.
 #define VCHECK(call)                                     \
     do {                                                 \
         cudaError_t e_ = (call);                         \
-        if (e_ != cudaSuccess) return VIPER_ECUDA;       \
+        if (e_ != cudaSuccess) {                         \
+            cudaGetLastError();                          \
+            return VIPER_ECUDA;                          \
+        }                                                \
     } while (0)
 
 template <class T>
@@ -828,6 +833,7 @@ int viper_scene_create(const viper_scene_desc *d, viper_scene **out)
     for (int r = 0; r < nr; ++r) s->h_rod_n[r] = s->h_off[r + 1] - s->h_off[r];
     auto fail = [&](int code) {
         viper_scene_destroy(s);
+        cudaGetLastError();  // as VCHECK
         return code;
     };
     if (d->stream) {
@@ -841,8 +847,8 @@ int viper_scene_create(const viper_scene_desc *d, viper_scene **out)
     if (cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming) != cudaSuccess) return fail(VIPER_ECUDA);
     if (cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess) return fail(VIPER_ECUDA);
     // mapped, so that the multi-scene step can write it from the device
-    if (cudaHostAlloc((void **)&s->h_err, 2 * sizeof(int), cudaHostAllocMapped) != cudaSuccess) return fail(VIPER_ECUDA);
-    s->h_err[0] = s->h_err[1] = 0;
+    if (cudaHostAlloc((void **)&s->h_err, 3 * sizeof(int), cudaHostAllocMapped) != cudaSuccess) return fail(VIPER_ECUDA);
+    s->h_err[0] = s->h_err[1] = s->h_err[2] = 0;
     if (cudaHostGetDevicePointer((void **)&s->d_herr, s->h_err, 0) != cudaSuccess) return fail(VIPER_ECUDA);
 
     // ---- rest data in FP64, caller order (Sec. 4 discretisation), kept for activation
@@ -1341,11 +1347,10 @@ int viper_skin(viper_scene *s, int n, const float *rest4, const int *idx4, const
     return cudaGetLastError() == cudaSuccess ? VIPER_OK : VIPER_ECUDA;
 }
 
-// Waits for the stream, on which the error word has been taken (take_error), and
-// reports it: overflow once; non-finite stays latched until a new state is set.
+// Reports the error word taken to h_err[1], the stream having been waited for:
+// overflow once; non-finite stays latched until a new state is set.
 static int taken_error(viper_scene *s)
 {
-    VCHECK(cudaStreamSynchronize(s->stream));
     s->latched |= s->h_err[1] | s->h_err[0];
     const int code = decode_err(s->latched);
     s->latched &= ERR_NONFINITE;
@@ -1359,6 +1364,7 @@ int viper_get_state(viper_scene *s, float *x4, float *v4, float *q4, float *w4)
     float *dst[4] = {x4, v4, q4, w4};
     StateArrays direct = {};
     bool any = false;
+    cudaGetLastError();  // an error left behind has been an earlier call's result
     for (int w = 0; w < 4; ++w) {
         if (!dst[w]) continue;
         const size_t bytes = sizeof(float4) * (size_t)(w < 2 ? s->nv : s->ns);
@@ -1378,11 +1384,10 @@ int viper_get_state(viper_scene *s, float *x4, float *v4, float *q4, float *w4)
         launch_state_out(s, w, s->stage4);
         VCHECK(cudaMemcpyAsync(dst[w], s->stage4, bytes, cudaMemcpyDefault, s->stream));
     }
-    if (any)
-        launch_state_out_all(s, direct);
-    else
-        launch_take_error(s);
+    if (any) launch_state_out_all(s, direct);
     VCHECK(cudaGetLastError());
+    if (!any) return viper_sync(s);
+    VCHECK(cudaStreamSynchronize(s->stream));
     return taken_error(s);
 }
 
@@ -1415,8 +1420,11 @@ int viper_set_state(viper_scene *s, const float *x4, const float *v4, const floa
 int viper_sync(viper_scene *s)
 {
     if (!s) return VIPER_EINVAL;
-    launch_take_error(s);
-    VCHECK(cudaGetLastError());
+    // by copies, as a kernel could not be launched while another device is current
+    VCHECK(cudaMemcpyAsync(s->h_err + 1, s->P.err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    VCHECK(cudaStreamSynchronize(s->stream));
+    if (s->h_err[1] && !(s->h_err[1] & ERR_NONFINITE))
+        VCHECK(cudaMemcpyAsync(s->P.err, s->h_err + 2, sizeof(int), cudaMemcpyHostToDevice, s->stream));
     return taken_error(s);
 }
 

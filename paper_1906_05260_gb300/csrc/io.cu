@@ -146,8 +146,6 @@ __device__ __forceinline__ void take_error(int *err, int *mirror)
     if (!(e & ERR_NONFINITE)) *err = 0;
 }
 
-__global__ void take_error_kernel(int *err, int *mirror) { take_error(err, mirror); }
-
 // All of the state in one launch, straight between the caller's device arrays
 // (null: left out) and the scene's: a thread per vertex, then per segment.  The
 // transfer is bound by its launches, not its bytes: eight copies and kernels,
@@ -215,12 +213,6 @@ void launch_state_out_all(viper_scene *s, const StateArrays &a)
 void launch_state_in_all(viper_scene *s, const StateArrays &a)
 {
     state_in_all_kernel<<<(s->nv + s->ns + 255) / 256, 256, 0, s->ls>>>(s->P, s->d_vperm, s->d_sperm, a);
-    s->launches++;
-}
-
-void launch_take_error(viper_scene *s)
-{
-    take_error_kernel<<<1, 1, 0, s->ls>>>(s->P.err, s->d_herr + 1);
     s->launches++;
 }
 

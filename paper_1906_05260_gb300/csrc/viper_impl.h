@@ -213,7 +213,7 @@ struct viper_scene {
     bool act_on = false;
     std::vector<int> u_xs_vert, u_xs_seg;  // bundle cross-section members, caller numbering
     // pinned, mapped host mirrors of the device error word: [0] written at the end of
-    // every frame (read without a stream sync), [1] when it is taken (take_error)
+    // every frame (read without a stream sync), [1] when it is taken (take_error); [2] stays zero
     int *h_err = nullptr;
     int *d_herr = nullptr;  // its device address
     void *self_table = nullptr;  // one-scene table of the multi-scene kernels (graph path)
@@ -285,7 +285,6 @@ struct StateArrays {
 };
 void launch_state_out_all(viper_scene *s, const StateArrays &a);  // and the error word to h_err[1] (take_error)
 void launch_state_in_all(viper_scene *s, const StateArrays &a);
-void launch_take_error(viper_scene *s);
 void launch_predicted_out(viper_scene *s, float4 *dst, float *rbar);
 int configure_rod_kernels(int smem_bytes);
 // scene helpers shared with the multi-scene step (capi.cu)
