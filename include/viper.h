@@ -364,8 +364,9 @@ int viper_contact_stats(viper_scene *scene, long long out[3]);
  *
  * Every kernel of the frame covers all scenes of the call: its grid is the
  * concatenation of the scenes' grids, so a frame of S substeps and I >= 1
- * iterations costs S (2 I + 3) + 3 launches (contacts, skinning) however
- * many scenes it carries.
+ * iterations costs S (2 I + 3) + 3 launches (contacts, skinning; three more
+ * a substep with a scene of more than 40,960 pills) however many scenes it
+ * carries.
  * Scenes with contacts or half-planes whose rods all fit the shared-memory
  * kernel (every scene whose rods are at most resident_max long) run the
  * contact-path sequence; such scenes without contacts run one launch for

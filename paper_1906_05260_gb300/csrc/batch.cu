@@ -9,11 +9,14 @@
 // scene computes the same thing alone and in a batch.
 //
 // Per substep, contact path (pills and/or half-planes), I >= 1 iterations:
-//   [velocity update of the previous substep + prediction + sweep 0] |
-//   grid (one CTA per scene: bounds, counts, scan, scatter) | pair search |
+//   velocity update of the previous substep + prediction |
+//   [grid (a cluster of CTAs per scene: cull, bounds, cut, counts, scan, scatter) |
+//   pair search] beside [sweep 0, on a second stream] |
 //   contact | {sweep | contact} x (I - 1)
-// and one velocity update after the last substep: S (2 I + 2) + 1 launches.
-// Without contacts: one launch for all substeps.  After the
+// and one velocity update after the last substep: S (2 I + 3) + 1 launches (three
+// more a substep where a scene is too large for the cluster's grid; without pills no
+// grid and search, and the update, the prediction and sweep 0 in one launch; bundles
+// add one).  Without contacts: one launch for all substeps.  After the
 // substeps one launch builds the skinning frames, hands the bone pose on and
 // mirrors the error word to the host; one more skins every mesh.
 //
@@ -690,9 +693,10 @@ __global__ void __launch_bounds__(256) batch_rod_first_kernel(BatchArgs A, int f
 // from the second sweep of a substep on, when the pair search found at least
 // two pairs per pill.  The sweep before such a pass writes them (48 bytes a
 // vertex); the same decision on both sides, from the pair count of the substep.
-// Scenes with few pairs do not pay for the packs; 45,000 pills of settled strands
-// (33 pairs a pill) take 7.7 ms a frame with this pass over up to four CTAs per SM,
-// 17.5 with 64 CTAs, scalar probes and no compaction.
+// A multi-scene frame without packs, with this rule and with packs always, in us: settled
+// strands, 13,000 pills (11 pairs a pill) 1,354, 1,324, 1,328, and 26,000 2,908, 2,680,
+// 2,670; falling, 26,000 pills (4) 1,102, 1,073, 1,068; 30 rigs of 40 muscles (next to
+// none) 1,902, 1,907, 1,922.
 constexpr int kPackPairs = 2;
 __device__ __forceinline__ bool packs_used(const Params &P, bool first_sweep)
 {
@@ -913,10 +917,11 @@ int resident_share(int want, int part, long long all)
 }
 
 // Groups of few pills do not fill the GPU with a thread per pill: several lanes
-// search a pill's neighbours (200 muscles, 6,910 pills, before the cull: 1,955 us
-// for two frames with one lane, 1,505 with two, 1,305 with four, 1,200 with eight;
-// strands and many scenes are fastest with one to four), and a contact CTA covers
-// fewer pills.
+// search a pill's neighbours, and a contact CTA covers fewer pills.  With one, two,
+// four and eight lanes, in us: 200 muscles, 6,910 pills, two frames 1,014, 977, 967,
+// 961 (few pills stay after the cull); a frame of settled strands, 14,300 pills, 1,512,
+// 1,330, 1,290, 1,276, and 19,500 1,788, 1,583, 1,552, 1,532; of falling ones, 9,100
+// pills, 719, 688, 672, 676, and 19,500 878, 826, 832, 834.
 constexpr int kSmallGroup = 20000, kEmitLanesSmall = 4, kContactPillsSmall = 64;
 constexpr int kMeshPerThread = 16;  // kLbsBatch vertices per round, 16 / kLbsBatch rounds
 
@@ -941,7 +946,7 @@ struct viper_batch {
     int cur = 0;
     std::vector<cudaEvent_t> ev;  // ordering after the scenes' streams
     cudaEvent_t ev_after = nullptr;
-    cudaStream_t side = nullptr;  // the broadphase branch of a sequence
+    cudaStream_t side = nullptr;  // the branch of a sequence with the first sweep
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     long long launches = 0;
 };
@@ -975,7 +980,7 @@ int stage_reserve(viper_batch::Stage &S, size_t bytes)
     return VIPER_OK;
 }
 
-// A second stream and two events for the broadphase branch of a sequence.
+// A second stream and two events for the branch of a sequence with the first sweep.
 struct Fork {
     cudaStream_t side;
     cudaEvent_t ev_fork, ev_join;
@@ -1093,7 +1098,7 @@ long long enqueue_sequence(const BatchArgs &A, const Shape &sh, int substeps, in
             launch_dependent(sh.small ? batch_emit_kernel<kEmitLanesSmall> : batch_emit_kernel<1>, tot[K_EMIT], 32 * kEmitWarpsB, 0, bs, A);
         });
     };
-    // the broadphase on a second branch beside the first sweep (not while profiling:
+    // the first sweep on a second branch beside the broadphase (not while profiling:
     // the per-class events bracket one stream)
     const bool forked = fork && fork->side && tot[K_PILL] > 0 && (!prof || prof->prof_class == PROF_NONE);
     auto contact = [&](int first) {
@@ -1223,9 +1228,13 @@ int run_group(viper_batch *B, const viper_batch_item *items, const std::vector<i
 
 }  // namespace
 
-// A larger scene alone runs the multi-kernel path, whose pair search and packs from
-// the first sweep on pay there (a frame of settled strands, 40,500 pills: 2.15 ms
-// against 2.45; falling, 27,000 pills: 1.05 against 1.07).
+// A larger scene alone runs the multi-kernel path: packs from the first sweep on and
+// passes over the whole GPU, but no cull.  The line is where rigs cross, which the cull
+// helps most (two frames, here and there, in us: 500 muscles, 18,061 pills, 1,515 and
+// 1,775; 620, 22,177 pills, 1,865 and 1,825; 190 bundles, 19,950 pills, 1,050 and 1,240;
+// 350, 36,750 pills, 1,295 and 1,373).  Strands cross at half of it (a frame, settled:
+// 10,400 pills 1,091 and 1,084, 19,500 1,514 and 1,428, 26,000 2,578 and 1,664; falling:
+// 7,150 pills 651 and 708, 19,500 829 and 739, 26,000 992 and 790).
 constexpr int kSelfMaxPills = 20000;
 
 bool self_batch_ok(const viper_scene *s)

@@ -9,11 +9,12 @@
 // coarsen the whole grid).  The grid is built with a count / exclusive-scan /
 // scatter pass that also copies each pill's sphere and group into cell order.
 // Candidate pairs are then built in parallel (the paper's extension of Green's
-// particle grid): a thread per pill tests the pills of its own cell after it
-// and those of the 13 forward neighbours (each neighbouring pair of cells is
-// visited once); a warp's hits are gathered in shared memory and written
-// together, one atomic reserving their slots.  The pair order inside the list
-// is not fixed, the pair set is; every consumer is order independent.
+// particle grid): a warp per oversized pill, then a thread per pill, which tests
+// the pills after it in its own row of cells and those of the four forward rows,
+// within its reach along x (five runs of the cell order; each pair is met
+// once); a warp's hits are gathered in shared memory and written together, one
+// atomic reserving their slots.  The pair order inside the list is not fixed,
+// the pair set is; every consumer is order independent.
 //
 // Contact handling (Sec. 7, Sec. 7.2): each candidate pair runs the
 // dichotomous narrowphase and, if the pills interpenetrate, one XPBD update of

@@ -842,7 +842,7 @@ __device__ __forceinline__ void rod_frame_item(const Params &P, int b, int subst
 // finish_prev, the prediction (Sec. 6) -- the start state kept in Xp / Qp,
 // the predicted world positions in Xpred when `world`, the half-plane
 // multipliers cleared -- then one colour sweep with fresh multipliers.
-// The same per-element arithmetic as finish_*_at, predict_*_at and rod_item.
+// The same per-element arithmetic as finish_*_at, predict_*_at and rod_run.
 __device__ __forceinline__ void rod_item_first(const Params &P, int b, bool finish_prev, float tau, bool world,
                                                float4 *smem)
 {
@@ -1097,7 +1097,7 @@ __device__ __forceinline__ void merge_bounds(const Params &P, float mn[3], float
 // thousands of pills in each cell.  The multi-kernel broadphase therefore
 // histograms the radii (16 bins per octave: the float's exponent and top four
 // mantissa bits) and sizes the cell for the cut radius below which all but at
-// most big_cap pills lie.  The pills above it sit in the cells like the others
+// most big_cap pills lie (the cluster's grid does the same).  The pills above it sit in the cells like the others
 // but are paired from their own side (emit_big).  The pair set is unchanged:
 // every candidate is still decided by spheres_overlap.
 constexpr unsigned int kRadBinBase = (127u - 20u) << 4;  // bin 0 starts at 2^-20
@@ -1177,7 +1177,7 @@ __device__ __forceinline__ void scatter_pill(const Params &P, int g, int cell, i
 }
 
 // Candidate pairs between one grid cell and one of its neighbours, by one
-// warp.  Every pair of pills whose cells are neighbours is visited exactly
+// warp (the frame solver's search).  Every pair of pills whose cells are neighbours is visited exactly
 // once: from the lower cell of the 13 "forward" neighbour offsets (dz = 1;
 // dz = 0, dy = 1; dz = dy = 0, dx = 1), and inside one cell from the pill at
 // the lower position.  Work unit u = 14 c + k pairs cell c with its forward
@@ -1359,9 +1359,11 @@ __device__ __forceinline__ bool spheres_overlap2(float4 na, float4 b)
 // end to end, four candidates a lane and step; the warp takes the longest walk's
 // number of steps.
 // L = 1 where the pills fill the GPU: settled strands (300,000 pills, 8.8
-// million pairs) take 216 us a search with the oversized pills, against 469 us
-// with fourteen lists each walked to the warp's longest and the oversized pills
-// tested against their whole list.  More lanes shorten the walk where they do not.
+// million pairs) took 216 us a search with the oversized pills when this walk was
+// made, in cubic cells (211 candidates a pill; make_grid_from's thinner ones leave 159),
+// against 469 us with fourteen lists each walked to the warp's longest and the
+// oversized pills tested against their whole list.  More lanes shorten the walk where
+// the pills do not fill the GPU.
 template <int L>
 __device__ __forceinline__ void emit_pills(const Params &P, const Grid &G, unsigned int big, int n, int warp,
                                            int nwarps, int *buf, int lane)

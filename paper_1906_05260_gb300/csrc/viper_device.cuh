@@ -40,14 +40,14 @@ __device__ __forceinline__ void add_to(float4 &p, V3 d)
 }
 
 // ---------------------------------------------------------------- approximate functions
-// The SFU's approximations in the forms that flush denormal operands and results to
-// zero: rsqrtf, __fdividef and the plain sqrt.approx test their operand for a
-// denormal, scale it up before and the result back after, three instructions in
-// a chain of a dozen.  The operands here are far from denormal (squared norms
-// of unit quaternions; sums of inverse masses, inertias and compliance terms, scaled
-// determinants; squared distances that only matter above 1e-24), where both
-// forms give the same bits.  16 rods, two frames 226 -> 200 us; 4,096 rods of 4 to 256
-// vertices 1,373 -> 1,270; a 200-muscle rig 1,003 -> 972.
+// The approximate root, inverse root and divide in the forms that flush subnormal
+// operands and results to zero (.ftz), with the same error bounds on normal numbers as
+// the forms that keep subnormals.  Roots, norms and denominators here are far from
+// subnormal (squared norms of unit quaternions; sums of inverse masses, inertias and
+// compliance terms, scaled determinants; squared distances that only matter above
+// 1e-24); a residual or increment below 1.2e-38 becomes zero.  On the chain of every
+// constraint: 16 rods, two frames 226 -> 200 us; 4,096 rods of 4 to 256 vertices
+// 1,373 -> 1,270; a 200-muscle rig 1,003 -> 972.
 __device__ __forceinline__ float rsqrt_approx(float x)
 {
     float r;

@@ -150,7 +150,7 @@ struct viper_scene {
     int n_rods = 0, nv = 0, ns = 0;
     cudaStream_t stream = nullptr;
     cudaStream_t ls = nullptr;     // stream the launchers enqueue on (stream, or side during a fork)
-    cudaStream_t side = nullptr;   // second branch: the broadphase runs beside the first rod sweep
+    cudaStream_t side = nullptr;   // second branch: the first rod sweep runs beside the broadphase
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     bool own_stream = false;
     int flags = 0, n_pins = 0, n_bones = 0, n_planes = 0;
@@ -293,7 +293,7 @@ bool scene_contact_path(const viper_scene *s);
 int scene_decode_err(int e);
 int scene_alloc(viper_scene *s, size_t bytes, void **out);  // device memory owned by the scene
 // The graph path of a scene whose rods all fit the shared-memory kernels (and,
-// with pills, whose grid fits one CTA): one frame of the multi-scene kernels
+// with pills, that has at most kSelfMaxPills of them): one frame of the multi-scene kernels
 // for this scene alone, captured on its stream (batch.cu).
 bool self_batch_ok(const viper_scene *s);
 int self_batch_capture(viper_scene *s, float dt, int substeps, int iterations, cudaGraph_t *graph,
